@@ -263,11 +263,13 @@ int lqcd_deo_apply_h16(lqcd_ctx *ctx, int out_parity, const void *in, const floa
  *   LQCD_PERSIST_REDUCTIONS=0  the solver iterations compute r -= alpha q,
  *                           ||r||^2 (every precision) and, in FP32 and FP16,
  *                           q = A p, <p, q> with one block per tile instead
- *                           of a grid of resident blocks that walk the tiles
- *                           (read once per process and device).
+ *                           of a grid of resident blocks that walk the tiles;
+ *                           small lattices run the same four kernels per
+ *                           iteration instead of many iterations in one
+ *                           cooperative launch (read once per process and
+ *                           device).
  * Every choice gives results within the documented tolerances; the
- * multi-RHS choices and the two forms of the reductions give identical
- * bits. */
+ * multi-RHS choices and the forms of the iteration give identical bits. */
 
 /* Launch configuration the autotuner chose for lqcd_deo_apply_ex(prec,
  * recon) on this context's lattice (the first such call times the candidates,

@@ -168,6 +168,8 @@ struct lqcd_ctx {
     lqcd::Workspace ws32;                  // FP32 phase of a hybrid mixed-precision solve
     std::vector<lqcd::Workspace> ref_ws;   // per-shift refinement jobs
     lqcd::GraphCache graph;
+    lqcd::DevBuf res_xch;     // flag words and published warp sums of the resident iteration
+    uint32_t res_tag = 0;     // last tag handed to a resident launch
     int *h_pinned = nullptr;  // pinned host words for halt/iteration polling
     double *h_pinned_d = nullptr;
     uint64_t launches = 0;    // library kernels launched on behalf of this context
@@ -248,6 +250,12 @@ int run_packed_until_halt(lqcd_ctx *c, const IterBatch<kMaxJobs> &B, int vp, int
 int mscg_solve_packed(lqcd_ctx *const *ctxs, int n, const double *mass, const double *const *shifts,
                       const int *n_shift, const double *tol, const double *const *b, double *const *x,
                       lqcd_solve_info *info);
+
+// resident.cu: iterations of the batch as cooperative launches until every
+// job halts; done = false: the batch does not take this path.
+constexpr int kResSteps = 256;   // iterations of one launch, at most
+template <int NJ>
+int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_iter, cudaStream_t s, bool &done);
 
 // helpers shared by solver.cu and mrhs.cu
 void k_res_nat1_ext(const Geom &g, const double2 *L, const double2 *x, double2 *t, int ntiles, cudaStream_t s);

@@ -616,9 +616,17 @@ template <int NJ>
 static int run_until_halt(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int chunk, int max_iter,
                           cudaStream_t s, std::vector<int> &halts)
 {
+    const int nj = B.njobs;
+    bool done = false;
+    if (int st = resident_run<NJ>(c, B, vp, lf, max_iter, s, done)) return st;
+    if (done) {
+        halts.assign(nj, 0);
+        for (int j = 0; j < nj; ++j)
+            LQCD_CUDA(cudaMemcpy(&halts[j], &B.job[j].st->halt, sizeof(int), cudaMemcpyDeviceToHost));
+        return LQCD_OK;
+    }
     cudaGraphExec_t exec = nullptr;
     if (int st = chunk_graph<NJ>(c, B, vp, lf, chunk, s, exec)) return st;
-    const int nj = B.njobs;
     // pinned status words: [2][nj] halts
     int *hs = c->h_pinned;
     const int max_chunks = max_iter / chunk + 4;
@@ -1109,7 +1117,7 @@ int job_finish(JobRun &J, cudaStream_t s)
     LQCD_CUDA(cudaMemcpyAsync(&O, J.P.st, sizeof O, cudaMemcpyDeviceToHost, s));
     LQCD_CUDA(cudaStreamSynchronize(s));
     if (O.halt == HALT_NAN) return fail(LQCD_ENAN, "NaN/Inf or breakdown in the multi-shift iteration");
-    if (O.halt == HALT_STALL) return fail(LQCD_ETIMEOUT, "a staged stencil wait for shared-memory link data ran out");
+    if (O.halt == HALT_STALL) return fail(LQCD_ETIMEOUT, "a bounded device wait of the iteration ran out");
     J.I.iters = O.iters;
     for (int i = 0; i < J.n_shift; ++i) J.I.shift_iters[i] = O.shift_iters[i];
     J.bytes += phase_bytes(J, O);

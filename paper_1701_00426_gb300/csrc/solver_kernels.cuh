@@ -184,74 +184,115 @@ __device__ inline void finalize_pq(SolverState *st, double pq)
 // finalize_pq on one warp, lane s = shift s (kMaxShifts == 32): every lane
 // loads its shift's scalars at once, the active list is compacted with a
 // ballot, and the recurrences of all shifts are updated in parallel.  Called
-// by warp 0 of the last block.
+// by warp 0 of the last block.  In two parts: alpha, which r -= alpha q waits
+// for, and the shifted coefficients, which only the shift updates need.
 static_assert(kMaxShifts == 32, "one lane per shift");
-__device__ inline void finalize_pq_warp(SolverState *st, double pq)
+struct PqCarry {
+    double alpha, alpha_old, beta_old, zo, zc, srel;
+    unsigned m;
+    int act;
+    bool ok;
+};
+
+__device__ __forceinline__ PqCarry finalize_pq_alpha(SolverState *st, double pq)
 {
     const int lane = threadIdx.x & 31;
+    PqCarry c;
     const int ns = st->n_shift;
-    const double rho = st->rho, alpha_old = st->alpha, beta_old = st->beta;
+    const double rho = st->rho;
+    c.alpha_old = st->alpha;
+    c.beta_old = st->beta;
     // every lane loads its shift's slots (kMaxShifts == 32) in one round trip
-    const int act = (lane < ns) ? st->active_next[lane] : 0;
-    const double zo = st->zeta[lane], zc = st->zeta_new[lane], srel = st->shift_rel[lane];
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, act);
-    const double alpha = rho / pq;
-    const bool ok = (pq > 0.0) && isfinite(alpha);
+    c.act = (lane < ns) ? st->active_next[lane] : 0;
+    c.zo = st->zeta[lane];
+    c.zc = st->zeta_new[lane];
+    c.srel = st->shift_rel[lane];
+    c.m = __ballot_sync(0xFFFFFFFFu, c.act);
+    c.alpha = rho / pq;
+    c.ok = (pq > 0.0) && isfinite(c.alpha);
     if (lane == 0) {
         st->last_sum = pq;
-        st->alpha_prev = alpha_old;
-        st->beta_prev = beta_old;
-        st->n_act = __popc(m);
-        if (ok) {
-            st->alpha = alpha;
-            st->alpha_df = split_scalar(alpha);
+        st->alpha_prev = c.alpha_old;
+        st->beta_prev = c.beta_old;
+        st->n_act = __popc(c.m);
+        if (c.ok) {
+            st->alpha = c.alpha;
+            st->alpha_df = split_scalar(c.alpha);
         } else {
             st->halt = HALT_NAN;
             st->nan_flag = 1;
         }
     }
-    if (!act) return;
+    return c;
+}
+
+__device__ __forceinline__ void finalize_pq_shifts(SolverState *st, const PqCarry &c)
+{
+    const int lane = threadIdx.x & 31;
+    if (!c.act) return;
     // rotate: zeta_prev <- zeta, zeta <- zeta_new
-    st->zeta_prev[lane] = zo;
-    st->zeta[lane] = zc;
-    st->act_list[__popc(m & ((1u << lane) - 1u))] = lane;
-    if (!ok) return;
-    const double den = alpha * beta_old * (zo - zc) + zo * alpha_old * (1.0 + srel * alpha);
-    const double zn = zc * zo * alpha_old / den;
+    st->zeta_prev[lane] = c.zo;
+    st->zeta[lane] = c.zc;
+    st->act_list[__popc(c.m & ((1u << lane) - 1u))] = lane;
+    if (!c.ok) return;
+    const double den =
+        c.alpha * c.beta_old * (c.zo - c.zc) + c.zo * c.alpha_old * (1.0 + c.srel * c.alpha);
+    const double zn = c.zc * c.zo * c.alpha_old / den;
     st->zeta_new[lane] = zn;
     st->zeta_new_df[lane] = split_scalar(zn);
-    st->alpha_s_df[lane] = split_scalar(alpha * zn / zc);
+    st->alpha_s_df[lane] = split_scalar(c.alpha * zn / c.zc);
+}
+
+__device__ inline void finalize_pq_warp(SolverState *st, double pq)
+{
+    const PqCarry c = finalize_pq_alpha(st, pq);
+    finalize_pq_shifts(st, c);
 }
 
 // finalize_rr on one warp: lane k handles the k-th active shift (beta_i and
 // the convergence test); lane 0 the base scalars and the halt decision.
-// Called by warp 0 of the last block.
-__device__ inline void finalize_rr_warp(SolverState *st, double rr)
+// Called by warp 0 of the last block.  In two parts: what does not depend on
+// ||r||^2, and the rest.
+struct RrCarry {
+    double rho, zn, ratio, tol2_b2, rel_stop2;
+    int s, its, iters, n_act, base, max_iter;
+};
+
+__device__ __forceinline__ RrCarry finalize_rr_begin(const SolverState *st)
+{
+    const int lane = threadIdx.x & 31;
+    RrCarry c;
+    c.rho = st->rho;
+    c.iters = st->iters + 1;
+    c.n_act = st->n_act;
+    c.tol2_b2 = st->tol2_b2;
+    // loaded up front so that lane 0's decisions wait on no further round trip
+    c.base = st->base;
+    c.max_iter = st->max_iter;
+    c.rel_stop2 = st->rel_stop2;
+    // lane l loads slot l of every per-shift array; lane k of the active list
+    // takes shift s = act_list[k]'s values by shuffle (one round trip)
+    c.s = st->act_list[lane] & (kMaxShifts - 1);
+    const double zc_l = st->zeta[lane], zn_l = st->zeta_new[lane];
+    const int it_l = st->shift_iters[lane];
+    const double zc = __shfl_sync(0xFFFFFFFFu, zc_l, c.s);
+    c.zn = __shfl_sync(0xFFFFFFFFu, zn_l, c.s);
+    c.its = __shfl_sync(0xFFFFFFFFu, it_l, c.s);
+    c.ratio = c.zn / zc;
+    return c;
+}
+
+__device__ __forceinline__ void finalize_rr_end(SolverState *st, const RrCarry &c, double rr)
 {
     const int lane = threadIdx.x & 31;
     const bool ok = isfinite(rr);
-    const double beta = rr / st->rho;
-    const int iters = st->iters + 1;
-    const int n_act = st->n_act;
-    const double tol2_b2 = st->tol2_b2;
-    // loaded up front so that lane 0's decisions wait on no further round trip
-    const int base = st->base, max_iter = st->max_iter;
-    const double rel_stop2 = st->rel_stop2;
-    // lane l loads slot l of every per-shift array; lane k of the active list
-    // takes shift s = act_list[k]'s values by shuffle (one round trip)
-    const int s = st->act_list[lane] & (kMaxShifts - 1);
-    const double zc_l = st->zeta[lane], zn_l = st->zeta_new[lane];
-    const int it_l = st->shift_iters[lane];
-    const double zc = __shfl_sync(0xFFFFFFFFu, zc_l, s);
-    const double zn = __shfl_sync(0xFFFFFFFFu, zn_l, s);
-    const int its = __shfl_sync(0xFFFFFFFFu, it_l, s);
+    const double beta = rr / c.rho;
     int open = 0;
-    if (ok && lane < n_act) {
-        const double ratio = zn / zc;
-        st->beta_s_df[s] = split_scalar(beta * ratio * ratio);
-        const bool conv = zn * zn * rr <= tol2_b2;
-        if (conv && its == 0) st->shift_iters[s] = iters;
-        st->active_next[s] = conv ? 0 : 1;
+    if (ok && lane < c.n_act) {
+        st->beta_s_df[c.s] = split_scalar(beta * c.ratio * c.ratio);
+        const bool conv = c.zn * c.zn * rr <= c.tol2_b2;
+        if (conv && c.its == 0) st->shift_iters[c.s] = c.iters;
+        st->active_next[c.s] = conv ? 0 : 1;
         open = !conv;
     }
     const int any = __any_sync(0xFFFFFFFFu, open);
@@ -269,16 +310,22 @@ __device__ inline void finalize_rr_warp(SolverState *st, double rr)
     }
     st->beta = beta;
     st->rho = rr;
-    st->iters = iters;
+    st->iters = c.iters;
     // the base direction must keep moving while any shift still iterates
-    if (any) st->active_next[base] = 1;
+    if (any) st->active_next[c.base] = 1;
     st->do_k4 = 1;
     if (!any)
         st->halt = HALT_CONVERGED;
-    else if (rel_stop2 > 0.0 && rr < rel_stop2)
+    else if (c.rel_stop2 > 0.0 && rr < c.rel_stop2)
         st->halt = HALT_RELIABLE;
-    else if (iters >= max_iter)
+    else if (c.iters >= c.max_iter)
         st->halt = HALT_MAXITER;
+}
+
+__device__ inline void finalize_rr_warp(SolverState *st, double rr)
+{
+    const RrCarry c = finalize_rr_begin(st);
+    finalize_rr_end(st, c, rr);
 }
 
 // beta, beta_i and the stopping decisions (FP64, one thread).
