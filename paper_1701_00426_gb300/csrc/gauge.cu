@@ -245,12 +245,8 @@ __device__ void staple_sum_dev(const LinkGeo &g, const typename Vec2T<T>::t *L, 
 // float4 per complex), products summed Dot2-style (common.cuh), so the
 // result carries ~48 significant bits on the FP32 pipes, which GB300 issues
 // 64 times faster than FP64.
-struct DC {
-    float2 re, im;
-};
-struct DM3 {
-    DC e[9];
-};
+using DC = Cplx<float2>;
+using DM3 = Mat3<float2>;
 
 __device__ __forceinline__ void dm_load(const float4 *__restrict__ L, int mu, int par, int idx, int Vh, DM3 &U)
 {
@@ -423,10 +419,214 @@ __global__ void __launch_bounds__(kGaugeThreads)
     for (int k = 0; k < 8; ++k) h[(size_t)k * Vh] = fma(-eps, f[k], h[(size_t)k * Vh]);
 }
 
-// U <- exp(i eps H) U in double-float: Z = i eps H scaled by 2^-k to
-// 1-norm <= 1/4 (scaling in FP64), Taylor series of degree 14 by Horner,
-// squared k times; the product is written to the IEEE master and to the
-// df64 copy.
+// ------------------------------------------------------------------ scalar arithmetic
+// One spelling for FP64 and double-float (float2 = hi, lo) reals.
+__device__ __forceinline__ double r_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float2 r_fma(float2 a, float2 b, float2 c) { return df_fma(a, b, c); }
+__device__ __forceinline__ double r_mul(double a, double b) { return a * b; }
+__device__ __forceinline__ float2 r_mul(float2 a, float2 b) { return df_mul(a, b); }
+__device__ __forceinline__ double r_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 r_add(float2 a, float2 b) { return df_add(a, b); }
+__device__ __forceinline__ double r_neg(double a) { return -a; }
+__device__ __forceinline__ float2 r_neg(float2 a) { return df_neg(a); }
+// times a power of two (exact)
+__device__ __forceinline__ double r_scale(double a, float p) { return a * (double)p; }
+__device__ __forceinline__ float2 r_scale(float2 a, float p) { return make_float2(a.x * p, a.y * p); }
+__device__ __forceinline__ float r_hi(double a) { return (float)a; }
+__device__ __forceinline__ float r_hi(float2 a) { return a.x; }
+template <class R> __device__ __forceinline__ R r_of(double v);
+template <> __device__ __forceinline__ double r_of<double>(double v) { return v; }
+template <> __device__ __forceinline__ float2 r_of<float2>(double v) { return f64_to_df_slow(v); }
+
+__device__ __forceinline__ void mm(const Mat3<double> &a, const Mat3<double> &b, Mat3<double> &c) { mat_mul(a, b, c); }
+__device__ __forceinline__ void mm(const DM3 &a, const DM3 &b, DM3 &c) { dm_mul<false>(a, b, c); }
+
+// 1 / n!, rounded to FP64 and split into double-float pairs
+constexpr int kExpDegMax = 20;
+constexpr double inv_fact(int n) { return n <= 1 ? 1.0 : inv_fact(n - 1) / n; }
+__constant__ double c_ifact64[kExpDegMax + 1] = {
+    inv_fact(0), inv_fact(1), inv_fact(2), inv_fact(3), inv_fact(4), inv_fact(5), inv_fact(6),
+    inv_fact(7), inv_fact(8), inv_fact(9), inv_fact(10), inv_fact(11), inv_fact(12), inv_fact(13),
+    inv_fact(14), inv_fact(15), inv_fact(16), inv_fact(17), inv_fact(18), inv_fact(19), inv_fact(20)};
+#define LQCD_IFACT_DF(n) {(float)inv_fact(n), (float)(inv_fact(n) - (double)(float)inv_fact(n))}
+__constant__ float2 c_ifact_df[kExpDegMax + 1] = {
+    LQCD_IFACT_DF(0), LQCD_IFACT_DF(1), LQCD_IFACT_DF(2), LQCD_IFACT_DF(3), LQCD_IFACT_DF(4), LQCD_IFACT_DF(5),
+    LQCD_IFACT_DF(6), LQCD_IFACT_DF(7), LQCD_IFACT_DF(8), LQCD_IFACT_DF(9), LQCD_IFACT_DF(10), LQCD_IFACT_DF(11),
+    LQCD_IFACT_DF(12), LQCD_IFACT_DF(13), LQCD_IFACT_DF(14), LQCD_IFACT_DF(15), LQCD_IFACT_DF(16),
+    LQCD_IFACT_DF(17), LQCD_IFACT_DF(18), LQCD_IFACT_DF(19), LQCD_IFACT_DF(20)};
+#undef LQCD_IFACT_DF
+template <class R> __device__ __forceinline__ R inv_factorial(int n);
+template <> __device__ __forceinline__ double inv_factorial<double>(int n) { return c_ifact64[n]; }
+template <> __device__ __forceinline__ float2 inv_factorial<float2>(int n) { return c_ifact_df[n]; }
+
+// ------------------------------------------------------------------ exponential
+// exp(iQ) of a traceless Hermitian Q.  By Cayley-Hamilton Q^3 = c1 Q + c0 with
+// c1 = Tr Q^2 / 2 and c0 = det Q, so every power series in Q is f0 + f1 Q +
+// f2 Q^2: the Taylor series runs on three complex coefficients instead of on
+// matrices (multiplying a + b Q + c Q^2 by iQ gives i c c0 + i (a + c c1) Q +
+// i b Q^2).  Horner with the coefficients 1/n!, 4 multiply-adds a step; no
+// division by eigenvalue differences, so nothing is lost near degenerate
+// eigenvalues.  |eigenvalue| <= sqrt(4 c1 / 3) =: r; Q is scaled by 2^-k to
+// r <= 1 and the result squared k times.  Degrees: the first term left out
+// is below 2^-64 (1/21! at r = 1).
+// Horner on matrices instead (17 products and the squarings from norm 1/4)
+// took, at 16^4: double-float link update 256 us, now 73 (20 us of memory
+// traffic; the rest double-float arithmetic); stout level 1884, now 851, and
+// with the block-matrix derivative the local pass of the force chain 5966,
+// now 1652 (both bound by the FP64 pipe).
+template <class R> struct Herm {
+    R d0, d1, d2;                    // diagonal
+    Cplx<R> a, b, c;                 // entries 01, 02, 12
+};
+template <class R> struct ExpF { R ar, ai, br, bi, cr, ci; };   // f0, f1, f2
+
+template <class R>
+__device__ __forceinline__ R norm2(const Cplx<R> &z) { return r_fma(z.re, z.re, r_mul(z.im, z.im)); }
+
+template <class R>
+__device__ __forceinline__ Herm<R> herm_square(const Herm<R> &q)
+{
+    Herm<R> s;
+    const R na = norm2(q.a), nb = norm2(q.b), nc = norm2(q.c);
+    s.d0 = r_fma(q.d0, q.d0, r_add(na, nb));
+    s.d1 = r_fma(q.d1, q.d1, r_add(na, nc));
+    s.d2 = r_fma(q.d2, q.d2, r_add(nb, nc));
+    const R t01 = r_add(q.d0, q.d1), t02 = r_add(q.d0, q.d2), t12 = r_add(q.d1, q.d2);
+    // 01: (d0 + d1) a + b conj(c);  02: (d0 + d2) b + a c;  12: (d1 + d2) c + conj(a) b
+    s.a.re = r_fma(t01, q.a.re, r_fma(q.b.re, q.c.re, r_mul(q.b.im, q.c.im)));
+    s.a.im = r_fma(t01, q.a.im, r_fma(q.b.im, q.c.re, r_neg(r_mul(q.b.re, q.c.im))));
+    s.b.re = r_fma(t02, q.b.re, r_fma(q.a.re, q.c.re, r_neg(r_mul(q.a.im, q.c.im))));
+    s.b.im = r_fma(t02, q.b.im, r_fma(q.a.re, q.c.im, r_mul(q.a.im, q.c.re)));
+    s.c.re = r_fma(t12, q.c.re, r_fma(q.a.re, q.b.re, r_mul(q.a.im, q.b.im)));
+    s.c.im = r_fma(t12, q.c.im, r_fma(q.a.re, q.b.im, r_neg(r_mul(q.a.im, q.b.re))));
+    return s;
+}
+
+template <class R>
+__device__ __forceinline__ R herm_det(const Herm<R> &q)
+{
+    // d0 (d1 d2 - |c|^2) - d1 |b|^2 - d2 |a|^2 + 2 Re(a c conj(b))
+    const R m = r_fma(q.d1, q.d2, r_neg(norm2(q.c)));
+    R t = r_fma(q.d0, m, r_neg(r_fma(q.d1, norm2(q.b), r_mul(q.d2, norm2(q.a)))));
+    const R xr = r_fma(q.a.re, q.c.re, r_neg(r_mul(q.a.im, q.c.im)));
+    const R xi = r_fma(q.a.re, q.c.im, r_mul(q.a.im, q.c.re));
+    const R y = r_fma(xr, q.b.re, r_mul(xi, q.b.im));
+    return r_add(t, r_add(y, y));
+}
+
+template <class R>
+__device__ __forceinline__ void herm_scale(Herm<R> &q, float p)
+{
+    q.d0 = r_scale(q.d0, p); q.d1 = r_scale(q.d1, p); q.d2 = r_scale(q.d2, p);
+    q.a = {r_scale(q.a.re, p), r_scale(q.a.im, p)};
+    q.b = {r_scale(q.b.re, p), r_scale(q.b.im, p)};
+    q.c = {r_scale(q.c.re, p), r_scale(q.c.im, p)};
+}
+
+// Q scaled to r <= 1 (k halvings), its square S, c0 and c1 of the scaled Q,
+// and the degree of the series.
+template <class R>
+struct ExpArg {
+    Herm<R> Q, S;
+    R c0, c1;
+    int k, deg;
+};
+
+template <class R>
+__device__ __forceinline__ ExpArg<R> exp_arg(const Herm<R> &q)
+{
+    ExpArg<R> X;
+    X.Q = q;
+    X.S = herm_square(q);
+    X.c1 = r_scale(r_add(X.S.d0, r_add(X.S.d1, X.S.d2)), 0.5f);
+    X.c0 = herm_det(q);
+    float r2 = 1.3333334f * r_hi(X.c1);
+    X.k = 0;
+    while (r2 > 1.f && X.k < 60) {
+        r2 *= 0.25f;
+        herm_scale(X.Q, 0.5f);
+        herm_scale(X.S, 0.25f);
+        X.c1 = r_scale(X.c1, 0.25f);
+        X.c0 = r_scale(X.c0, 0.125f);
+        ++X.k;
+    }
+    X.deg = r2 <= 1.f / 256 ? 10 : (r2 <= 1.f / 16 ? 13 : kExpDegMax);
+    return X;
+}
+
+template <class R>
+__device__ __forceinline__ ExpF<R> exp_coef(const ExpArg<R> &X)
+{
+    ExpF<R> f;
+    const R zero = r_of<R>(0.0);
+    f.ar = inv_factorial<R>(X.deg);
+    f.ai = f.br = f.bi = f.cr = f.ci = zero;
+#pragma unroll 1
+    for (int n = X.deg - 1; n >= 0; --n) {
+        const R ar = r_fma(r_neg(f.ci), X.c0, inv_factorial<R>(n)), ai = r_mul(f.cr, X.c0);
+        const R br = r_neg(r_fma(f.ci, X.c1, f.ai)), bi = r_fma(f.cr, X.c1, f.ar);
+        f.cr = r_neg(f.bi);
+        f.ci = f.br;
+        f.ar = ar;
+        f.ai = ai;
+        f.br = br;
+        f.bi = bi;
+    }
+    return f;
+}
+
+// E = f0 + f1 Q + f2 S for the entry pair (ij, ji) with Q_ij = q, S_ij = s
+template <class R>
+__device__ __forceinline__ void exp_pair(const ExpF<R> &f, const Cplx<R> &q, const Cplx<R> &s, Cplx<R> &u, Cplx<R> &l)
+{
+    const R t1 = r_fma(f.br, q.re, r_mul(f.cr, s.re)), t2 = r_fma(f.bi, q.im, r_mul(f.ci, s.im));
+    const R t3 = r_fma(f.br, q.im, r_mul(f.cr, s.im)), t4 = r_fma(f.bi, q.re, r_mul(f.ci, s.re));
+    u = {r_add(t1, r_neg(t2)), r_add(t3, t4)};
+    l = {r_add(t1, t2), r_add(t4, r_neg(t3))};
+}
+
+template <class R>
+__device__ __forceinline__ void exp_matrix(const ExpArg<R> &X, const ExpF<R> &f, Mat3<R> &E)
+{
+    E.e[0] = {r_fma(f.br, X.Q.d0, r_fma(f.cr, X.S.d0, f.ar)), r_fma(f.bi, X.Q.d0, r_fma(f.ci, X.S.d0, f.ai))};
+    E.e[4] = {r_fma(f.br, X.Q.d1, r_fma(f.cr, X.S.d1, f.ar)), r_fma(f.bi, X.Q.d1, r_fma(f.ci, X.S.d1, f.ai))};
+    E.e[8] = {r_fma(f.br, X.Q.d2, r_fma(f.cr, X.S.d2, f.ar)), r_fma(f.bi, X.Q.d2, r_fma(f.ci, X.S.d2, f.ai))};
+    exp_pair(f, X.Q.a, X.S.a, E.e[1], E.e[3]);
+    exp_pair(f, X.Q.b, X.S.b, E.e[2], E.e[6]);
+    exp_pair(f, X.Q.c, X.S.c, E.e[5], E.e[7]);
+}
+
+// E = exp(iQ)
+template <class R>
+__device__ __forceinline__ void exp_herm(const Herm<R> &Q, Mat3<R> &E)
+{
+    const ExpArg<R> X = exp_arg(Q);
+    const ExpF<R> f = exp_coef(X);
+    exp_matrix(X, f, E);
+#pragma unroll 1
+    for (int q = 0; q < X.k; ++q) {
+        Mat3<R> T;
+        mm(E, E, T);
+        E = T;
+    }
+}
+
+// t H of 8 reals
+template <class R, class T>
+__device__ __forceinline__ Herm<R> herm_from(const T (&h)[8], T t)
+{
+    Herm<R> q;
+    q.d0 = r_of<R>((double)(t * h[0]));
+    q.d1 = r_of<R>((double)(t * h[1]));
+    q.d2 = r_of<R>((double)(-t * (h[0] + h[1])));
+    q.a = {r_of<R>((double)(t * h[2])), r_of<R>((double)(t * h[3]))};
+    q.b = {r_of<R>((double)(t * h[4])), r_of<R>((double)(t * h[5]))};
+    q.c = {r_of<R>((double)(t * h[6])), r_of<R>((double)(t * h[7]))};
+    return q;
+}
+
+// U <- exp(i eps H) U in double-float (eps H formed in FP64); the product is
+// written to the IEEE master and to the df64 copy.
 __global__ void __launch_bounds__(kGaugeThreads)
     k_gauge_link_update_df(int Vh, double2 *__restrict__ nat, float4 *__restrict__ Ldf,
                            const double *__restrict__ mom, double eps)
@@ -439,60 +639,15 @@ __global__ void __launch_bounds__(kGaugeThreads)
     const double *hp = mom + (size_t)(mp * 8) * Vh + i;
 #pragma unroll
     for (int k = 0; k < 8; ++k) h[k] = hp[(size_t)k * Vh];
-    // 1-norm of H (columns), in FP64
-    const double h22 = -h[0] - h[1];
-    const double a01 = sqrt(h[2] * h[2] + h[3] * h[3]), a02 = sqrt(h[4] * h[4] + h[5] * h[5]),
-                 a12 = sqrt(h[6] * h[6] + h[7] * h[7]);
-    double nrm = fmax(fabs(h[0]) + a01 + a02, fmax(a01 + fabs(h[1]) + a12, a02 + a12 + fabs(h22)));
-    nrm *= fabs(eps);
-    int k = 0;
-    double sc = eps;
-    while (nrm > 0.25 && k < 60) {
-        nrm *= 0.5;
-        sc *= 0.5;
-        ++k;
-    }
-    // Z = i sc H: Z_ab = i sc H_ab -> re = -sc Im H_ab, im = sc Re H_ab
-    DM3 Z;
-    {
-        const double hr[9] = {h[0], h[2], h[4], h[2], h[1], h[6], h[4], h[6], h22};
-        const double hi[9] = {0.0, h[3], h[5], -h[3], 0.0, h[7], -h[5], -h[7], 0.0};
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            Z.e[q].re = f64_to_df_slow(-sc * hi[q]);
-            Z.e[q].im = f64_to_df_slow(sc * hr[q]);
-        }
-    }
-    DM3 R, ZR;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        R.e[q].re = make_float2(q % 4 == 0 ? 1.f : 0.f, 0.f);
-        R.e[q].im = make_float2(0.f, 0.f);
-    }
-#pragma unroll 1
-    for (int n = 14; n >= 1; --n) {
-        dm_mul<false>(Z, R, ZR);
-        const float2 inv = f64_to_df_slow(1.0 / n);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            R.e[q].re = df_mul(inv, ZR.e[q].re);
-            R.e[q].im = df_mul(inv, ZR.e[q].im);
-            if (q % 4 == 0) R.e[q].re = df_add(R.e[q].re, make_float2(1.f, 0.f));
-        }
-    }
-#pragma unroll 1
-    for (int q = 0; q < k; ++q) {
-        dm_mul<false>(R, R, ZR);
-        R = ZR;
-    }
-    DM3 U;
+    DM3 E, U, W;
+    exp_herm(herm_from<float2>(h, eps), E);
     dm_load(Ldf, mp >> 1, mp & 1, i, Vh, U);
-    dm_mul<false>(R, U, ZR);
+    dm_mul<false>(E, U, W);
     double2 *pn = nat + (size_t)(mp * 9) * Vh + i;
     float4 *pd = Ldf + (size_t)(mp * 9) * Vh + i;
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
-        const float2 re = ZR.e[c].re, im = ZR.e[c].im;
+        const float2 re = W.e[c].re, im = W.e[c].im;
         pn[(size_t)c * Vh] = make_double2(df_to_f64(re), df_to_f64(im));
         pd[(size_t)c * Vh] = make_float4(re.x, re.y, im.x, im.y);
     }
@@ -565,11 +720,13 @@ __global__ void __launch_bounds__(kGaugeThreads)
     for (int k = 0; k < 8; ++k) h[(size_t)k * Vh] = fma(-eps, f[k], h[(size_t)k * Vh]);
 }
 
-// E = exp(i t H): Z = i t H scaled by 2^-k to 1-norm <= 1/4, Taylor series of
-// degree 16 (FP64) or 9 (FP32), squared k times.
-template <class T>
-__device__ __forceinline__ void exp_iH_dev(const Mat3<T> &H, T t, Mat3<T> &E)
+// E = exp(i t H) in FP32: Z = i t H scaled by 2^-k to 1-norm <= 1/4, Taylor
+// series of degree 9 on the matrix, squared k times.  exp_herm rounds
+// differently (2e-7 after 40 steps), and an FP32 trajectory is kept
+// reproducible to the bit; the update is 8 % of an FP32 step.
+__device__ __forceinline__ void exp_iH_f32(const Mat3<float> &H, float t, Mat3<float> &E)
 {
+    using T = float;
     T nrm = 0;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -590,7 +747,7 @@ __device__ __forceinline__ void exp_iH_dev(const Mat3<T> &H, T t, Mat3<T> &E)
 #pragma unroll
     for (int q = 0; q < 9; ++q) Z.e[q] = {-sc * H.e[q].im, sc * H.e[q].re};
     // Horner: E = I + Z (I + Z/2 (I + Z/3 (... (I + Z/n))))
-    constexpr int deg = sizeof(T) == 8 ? 16 : 9;
+    constexpr int deg = 9;
     Mat3<T> R;
 #pragma unroll
     for (int q = 0; q < 9; ++q) R.e[q] = {(q % 4 == 0) ? T(1) : T(0), T(0)};
@@ -624,9 +781,14 @@ __global__ void __launch_bounds__(kGaugeThreads)
     const T *hp = mom + (size_t)(mp * 8) * Vh + i;
 #pragma unroll
     for (int k = 0; k < 8; ++k) h[k] = hp[(size_t)k * Vh];
-    Mat3<T> H, E, U, R;
-    herm_unpack(h, H);
-    exp_iH_dev(H, eps, E);
+    Mat3<T> E, U, R;
+    if constexpr (sizeof(T) == 4) {
+        Mat3<T> H;
+        herm_unpack(h, H);
+        exp_iH_f32(H, eps, E);
+    } else {
+        exp_herm(herm_from<T>(h, eps), E);
+    }
     typename Vec2T<T>::t *p = L + (size_t)(mp * 9) * Vh + i;
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
@@ -980,85 +1142,125 @@ __device__ __forceinline__ void stout_C(const LinkGeo &g, const double2 *L, cons
 }
 
 // Q from C and U (Hermitian, traceless)
-__device__ __forceinline__ void stout_Q(const Mat3<double> &C, const Mat3<double> &U, Mat3<double> &Q)
+__device__ __forceinline__ Herm<double> stout_Q(const Mat3<double> &C, const Mat3<double> &U)
 {
     Mat3<double> Om;
     mat_mul_dag(C, U, Om);
     // Q_ij = (i/2)(conj(Om_ji) - Om_ij):  re = (Om_ij.im + Om_ji.im)/2, im = (Om_ji.re - Om_ij.re)/2
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-            Q.e[i * 3 + j] = {0.5 * (Om.e[i * 3 + j].im + Om.e[j * 3 + i].im),
-                              0.5 * (Om.e[j * 3 + i].re - Om.e[i * 3 + j].re)};
-    const double tr = (Q.e[0].re + Q.e[4].re + Q.e[8].re) / 3.0;
-    Q.e[0].re -= tr;
-    Q.e[4].re -= tr;
-    Q.e[8].re -= tr;
+    auto q = [&](int ij, int ji) -> Cplx<double> {
+        return {0.5 * (Om.e[ij].im + Om.e[ji].im), 0.5 * (Om.e[ji].re - Om.e[ij].re)};
+    };
+    const double tr = (Om.e[0].im + Om.e[4].im + Om.e[8].im) / 3.0;
+    Herm<double> Q;
+    Q.d0 = Om.e[0].im - tr;
+    Q.d1 = Om.e[4].im - tr;
+    Q.d2 = Om.e[8].im - tr;
+    Q.a = q(1, 3);
+    Q.b = q(2, 6);
+    Q.c = q(5, 7);
+    return Q;
 }
 
-// E = exp(X) and D = d/dt exp(X + t A) at t = 0, from the block matrix
-// B = [[X, A], [0, X]], exp(B) = [[E, D], [0, E]]: B scaled by 2^-k to
-// 1-norm <= 1/4 (the norm of X bounds the scaling; A scales with it),
-// Horner on the block form (P <- 1 + X P / n, R <- (X R + A P) / n, degree
-// 18), then k block squarings (P, R) <- (P P, P R + R P).
-__device__ void exp_frechet_dev(const Mat3<double> &X, const Mat3<double> &A, Mat3<double> &E, Mat3<double> &D)
+// complex helpers (FP64)
+using Cd = Cplx<double>;
+__device__ __forceinline__ Cd c_mul(Cd a, Cd b) { return {fma(a.re, b.re, -a.im * b.im), fma(a.re, b.im, a.im * b.re)}; }
+__device__ __forceinline__ Cd c_fma(Cd a, Cd b, Cd c)
 {
-    // D is linear in A: run with A / ||A||_1 and scale D back
-    double nx = 0.0, na = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        double c = 0.0, ca = 0.0;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            c += hypot(X.e[i * 3 + j].re, X.e[i * 3 + j].im);
-            ca += hypot(A.e[i * 3 + j].re, A.e[i * 3 + j].im);
-        }
-        nx = fmax(nx, c);
-        na = fmax(na, ca);
+    return {fma(a.re, b.re, fma(-a.im, b.im, c.re)), fma(a.re, b.im, fma(a.im, b.re, c.im))};
+}
+
+__device__ __forceinline__ void herm_matrix(const Herm<double> &q, Mat3<double> &M)
+{
+    M.e[0] = {q.d0, 0.0};
+    M.e[4] = {q.d1, 0.0};
+    M.e[8] = {q.d2, 0.0};
+    M.e[1] = q.a;
+    M.e[3] = {q.a.re, -q.a.im};
+    M.e[2] = q.b;
+    M.e[6] = {q.b.re, -q.b.im};
+    M.e[5] = q.c;
+    M.e[7] = {q.c.re, -q.c.im};
+}
+
+// Tr(Q B) for a Hermitian Q
+__device__ __forceinline__ Cd herm_trace(const Herm<double> &q, const Mat3<double> &B)
+{
+    Cd t = {fma(q.d0, B.e[0].re, fma(q.d1, B.e[4].re, q.d2 * B.e[8].re)),
+            fma(q.d0, B.e[0].im, fma(q.d1, B.e[4].im, q.d2 * B.e[8].im))};
+    auto pair = [&](const Cd &z, int ij, int ji) {  // Q_ij B_ji + conj(Q_ij) B_ij
+        t = c_fma(z, B.e[ji], t);
+        t = c_fma(Cd{z.re, -z.im}, B.e[ij], t);
+    };
+    pair(q.a, 1, 3);
+    pair(q.b, 2, 6);
+    pair(q.c, 5, 7);
+    return t;
+}
+
+// E = exp(iQ) and D = d/dt exp(iQ + t A) at t = 0.  With A = i (B + beta 1),
+// Tr B = 0: D = i beta E + df0 + df1 Q + df2 Q^2 + f1 B + f2 (Q B + B Q), where
+// df_j = (df_j/dc1) Tr(Q B) + (df_j/dc0) Tr(Q^2 B) (the differentials of
+// c1 = Tr Q^2 / 2 and c0 = Tr Q^3 / 3 along a traceless B).  The series and its
+// two derivatives run on scalars (exp_coef's recurrence, differentiated);
+// what is left of the 66 matrix products of a block-matrix series are Q B
+// and B Q.  k halvings are undone by (E, D) <- (E E, E D + D E).
+__device__ void exp_frechet_dev(const Herm<double> &Q, const Mat3<double> &A, Mat3<double> &E, Mat3<double> &D)
+{
+    const ExpArg<double> X = exp_arg(Q);
+    // value (a, b, c), derivative by c1 (p, q, r) and by c0 (x, y, z)
+    Cd a = {inv_factorial<double>(X.deg), 0.0}, b = {0, 0}, c = {0, 0};
+    Cd p = {0, 0}, q = {0, 0}, r = {0, 0}, x = {0, 0}, y = {0, 0}, z = {0, 0};
+    auto times_i = [](Cd v) -> Cd { return {-v.im, v.re}; };
+    auto axpy = [](double s, Cd v, Cd w) -> Cd { return {fma(s, v.re, w.re), fma(s, v.im, w.im)}; };
+#pragma unroll 1
+    for (int n = X.deg - 1; n >= 0; --n) {
+        const Cd a1 = times_i({c.re * X.c0, c.im * X.c0}), b1 = times_i(axpy(X.c1, c, a)), c1 = times_i(b);
+        const Cd p1 = times_i({r.re * X.c0, r.im * X.c0});
+        const Cd q1 = times_i(axpy(X.c1, r, {p.re + c.re, p.im + c.im})), r1 = times_i(q);
+        const Cd x1 = times_i(axpy(X.c0, z, c)), y1 = times_i(axpy(X.c1, z, x)), z1 = times_i(y);
+        a = {a1.re + inv_factorial<double>(n), a1.im};
+        b = b1; c = c1;
+        p = p1; q = q1; r = r1;
+        x = x1; y = y1; z = z1;
     }
-    const double an = na > 0.0 ? 1.0 / na : 0.0;
-    double nrm = nx + (na > 0.0 ? 1.0 : 0.0);
-    int k = 0;
-    while (nrm > 0.25 && k < 60) {
-        nrm *= 0.5;
-        ++k;
-    }
-    const double sc = ldexp(1.0, -k);
-    Mat3<double> Xs, As, P, R;
+    const ExpF<double> f = {a.re, a.im, b.re, b.im, c.re, c.im};
+    exp_matrix(X, f, E);
+    // -i A / 2^k = B + beta 1
+    const double sc = ldexp(1.0, -X.k);
+    Mat3<double> B, H, T;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        Xs.e[q] = {sc * X.e[q].re, sc * X.e[q].im};
-        As.e[q] = {sc * an * A.e[q].re, sc * an * A.e[q].im};
-        P.e[q] = {(q % 4 == 0) ? 1.0 : 0.0, 0.0};
-        R.e[q] = {0.0, 0.0};
+    for (int e = 0; e < 9; ++e) B.e[e] = {sc * A.e[e].im, -sc * A.e[e].re};
+    const Cd beta = {(B.e[0].re + B.e[4].re + B.e[8].re) / 3.0, (B.e[0].im + B.e[4].im + B.e[8].im) / 3.0};
+#pragma unroll
+    for (int e = 0; e < 9; e += 4) B.e[e] = {B.e[e].re - beta.re, B.e[e].im - beta.im};
+    const Cd t1 = herm_trace(X.Q, B), t0 = herm_trace(X.S, B);
+    const Cd g0 = c_fma(p, t1, c_mul(x, t0)), g1 = c_fma(q, t1, c_mul(y, t0)), g2 = c_fma(r, t1, c_mul(z, t0));
+    const Cd ib = times_i(beta);
+    herm_matrix(X.Q, H);
+    mat_mul(H, B, T);
+    mat_mul(B, H, D);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        const Cd g = {T.e[e].re + D.e[e].re, T.e[e].im + D.e[e].im};
+        Cd v = c_fma(c, g, c_fma(b, B.e[e], c_mul(ib, E.e[e])));
+        v = c_fma(g1, H.e[e], v);
+        D.e[e] = v;
+    }
+    herm_matrix(X.S, H);
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        D.e[e] = c_fma(g2, H.e[e], D.e[e]);
+        if (e % 4 == 0) D.e[e] = {D.e[e].re + g0.re, D.e[e].im + g0.im};
     }
 #pragma unroll 1
-    for (int n = 18; n >= 1; --n) {
-        Mat3<double> XP, XR, AP;
-        mat_mul(Xs, P, XP);
-        mat_mul(Xs, R, XR);
-        mat_mul(As, P, AP);
-        const double inv = 1.0 / n;
+    for (int k = 0; k < X.k; ++k) {
+        mat_mul(E, D, T);
+        mat_mul(D, E, H);
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            P.e[q] = {((q % 4 == 0) ? 1.0 : 0.0) + inv * XP.e[q].re, inv * XP.e[q].im};
-            R.e[q] = {inv * (XR.e[q].re + AP.e[q].re), inv * (XR.e[q].im + AP.e[q].im)};
-        }
+        for (int e = 0; e < 9; ++e) D.e[e] = {T.e[e].re + H.e[e].re, T.e[e].im + H.e[e].im};
+        mat_mul(E, E, T);
+        E = T;
     }
-#pragma unroll 1
-    for (int q = 0; q < k; ++q) {
-        Mat3<double> PP, PR, RP;
-        mat_mul(P, P, PP);
-        mat_mul(P, R, PR);
-        mat_mul(R, P, RP);
-        P = PP;
-#pragma unroll
-        for (int c = 0; c < 9; ++c) R.e[c] = {PR.e[c].re + RP.e[c].re, PR.e[c].im + RP.e[c].im};
-    }
-    E = P;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) D.e[c] = {na * R.e[c].re, na * R.e[c].im};
 }
 
 __device__ __forceinline__ void store_link_soa(double2 *L, int mu, int P, int i, int Vh, const Mat3<double> &U)
@@ -1080,11 +1282,10 @@ __global__ void __launch_bounds__(kGaugeThreads)
     const int mu = mp >> 1, P = mp & 1;
     int x[4];
     coords_of(g, P, i, x);
-    Mat3<double> C, U, Q, E, R;
+    Mat3<double> C, U, E, R;
     stout_C(g, Lin, x, mu, rho, C);
     load_link_soa<double>(Lin, mu, P, i, Vh, U);
-    stout_Q(C, U, Q);
-    exp_iH_dev(Q, 1.0, E);
+    exp_herm(stout_Q(C, U), E);
     mat_mul(E, U, R);
     store_link_soa(Lout, mu, P, i, Vh, R);
 }
@@ -1107,28 +1308,25 @@ __global__ void __launch_bounds__(kGaugeThreads)
     const int mu = mp >> 1, P = mp & 1;
     int x[4];
     coords_of(g, P, i, x);
-    Mat3<double> C, U, Q, E, D, W, S, iQ, F;
+    Mat3<double> C, U, E, D, W, S, F;
     stout_C(g, L, x, mu, rho, C);
     load_link_soa<double>(L, mu, P, i, Vh, U);
-    stout_Q(C, U, Q);
+    const Herm<double> Q = stout_Q(C, U);
     double h[8];
     const double *hp = Fp + (size_t)(mp * 8) * Vh + i;
 #pragma unroll
     for (int k = 0; k < 8; ++k) h[k] = hp[(size_t)k * Vh];
     herm_unpack(h, F);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) iQ.e[q] = {-Q.e[q].im, Q.e[q].re};
-    exp_iH_dev(Q, 1.0, E);
+    exp_herm(Q, E);
     mat_mul(E, U, W);  // U'
     // S = -i U'^dag F
-    Mat3<double> Wd = W;
-    mat_dag(Wd);
-    mat_mul(Wd, F, S);
+    mat_dag(W);
+    mat_mul(W, F, S);
 #pragma unroll
     for (int q = 0; q < 9; ++q) S.e[q] = {S.e[q].im, -S.e[q].re};
-    Mat3<double> US, E2;
+    Mat3<double> US;
     mat_mul(U, S, US);
-    exp_frechet_dev(iQ, US, E2, D);
+    exp_frechet_dev(Q, US, E, D);
     // L = (D - D^dag)/2 - Tr(D - D^dag)/6
     Mat3<double> Lm;
 #pragma unroll
@@ -1161,7 +1359,8 @@ __global__ void __launch_bounds__(kGaugeThreads)
 //   U_mu(y+l) U_l(y+mu)^dag M_mu(y)            U_mu(y-mu+l)^dag U_l(y-mu)^dag M_mu(y-mu)^dag
 //   M_mu(y+l)^dag U_l(y+mu)^dag U_mu(y)^dag    M_mu(y+l-mu) U_l(y-mu)^dag U_mu(y-mu)
 //   U_nu(y-nu+l)^dag M_l(y-nu) U_nu(y-nu)      U_nu(y+l) M_l(y+nu) U_nu(y)^dag
-// adds the link's own terms Gl and writes the force on the link,
+// (the terms that end in the same link share its product: 10 products for the
+// six terms instead of 12; 1980 -> 1692 us at 16^4, FP64 pipe), adds the link's own terms Gl and writes the force on the link,
 //   F = traceless part of (i/2)(U G - G^dag U^dag), as 8 reals.
 __global__ void __launch_bounds__(kGaugeThreads)
     k_stout_gather(LinkGeo g, const double2 *__restrict__ L, const double2 *__restrict__ M,
@@ -1187,51 +1386,42 @@ __global__ void __launch_bounds__(kGaugeThreads)
         int em[4] = {0, 0, 0, 0};
         em[m] = 1;
         Mat3<double> a, b, c, t1, t2;
-        // U_m(y+l) U_l(y+m)^dag M_m(y)
+        // upper: U_m(y+l) U_l(y+m)^dag M_m(y)
+        //        + [ U_m(y+l) M_l(y+m) + M_m(y+l)^dag U_l(y+m)^dag ] U_m(y)^dag
         link_at<double>(g, L, y, el[0], el[1], el[2], el[3], m, a);
+        link_at<double>(g, M, y, em[0], em[1], em[2], em[3], l, c);
+        mat_mul(a, c, t2);
         link_at<double>(g, L, y, em[0], em[1], em[2], em[3], l, b);
         mat_mul_dag(a, b, t1);
         link_at<double>(g, M, y, 0, 0, 0, 0, m, c);
-        mat_mul(t1, c, t2);
-        mat_axpy(1.0, t2, acc);
-        // U_m(y-m+l)^dag U_l(y-m)^dag M_m(y-m)^dag = (M_m(y-m) U_l(y-m) U_m(y-m+l))^dag
-        link_at<double>(g, M, y, -em[0], -em[1], -em[2], -em[3], m, c);
-        link_at<double>(g, L, y, -em[0], -em[1], -em[2], -em[3], l, b);
-        mat_mul(c, b, t1);
-        link_at<double>(g, L, y, el[0] - em[0], el[1] - em[1], el[2] - em[2], el[3] - em[3], m, a);
-        mat_mul(t1, a, t2);
-        mat_dag(t2);
-        mat_axpy(1.0, t2, acc);
-        // M_m(y+l)^dag U_l(y+m)^dag U_m(y)^dag = (U_m(y) U_l(y+m) M_m(y+l))^dag
-        link_at<double>(g, L, y, 0, 0, 0, 0, m, a);
-        link_at<double>(g, L, y, em[0], em[1], em[2], em[3], l, b);
-        mat_mul(a, b, t1);
+        mat_mul(t1, c, a);
+        mat_axpy(1.0, a, acc);
+        mat_dag(b);
         link_at<double>(g, M, y, el[0], el[1], el[2], el[3], m, c);
-        mat_mul(t1, c, t2);
+        mat_dag(c);
+        mat_mul(c, b, t1);
+        mat_axpy(1.0, t1, t2);
+        link_at<double>(g, L, y, 0, 0, 0, 0, m, b);
+        mat_mul_dag(t2, b, t1);
+        mat_axpy(1.0, t1, acc);
+        // lower: (M_m(y-m) U_l(y-m) U_m(y-m+l))^dag
+        //        + [ M_m(y+l-m) U_l(y-m)^dag + U_m(y-m+l)^dag M_l(y-m) ] U_m(y-m)
+        link_at<double>(g, L, y, el[0] - em[0], el[1] - em[1], el[2] - em[2], el[3] - em[3], m, a);
+        link_at<double>(g, L, y, -em[0], -em[1], -em[2], -em[3], l, b);
+        mat_mul(b, a, t1);
+        link_at<double>(g, M, y, -em[0], -em[1], -em[2], -em[3], m, c);
+        mat_mul(c, t1, t2);
         mat_dag(t2);
         mat_axpy(1.0, t2, acc);
-        // M_m(y+l-m) U_l(y-m)^dag U_m(y-m)
-        link_at<double>(g, M, y, el[0] - em[0], el[1] - em[1], el[2] - em[2], el[3] - em[3], m, c);
-        link_at<double>(g, L, y, -em[0], -em[1], -em[2], -em[3], l, b);
-        mat_mul_dag(c, b, t1);
-        link_at<double>(g, L, y, -em[0], -em[1], -em[2], -em[3], m, a);
-        mat_mul(t1, a, t2);
-        mat_axpy(1.0, t2, acc);
-        // (m plays nu) U_m(y-m+l)^dag M_l(y-m) U_m(y-m)
-        link_at<double>(g, L, y, el[0] - em[0], el[1] - em[1], el[2] - em[2], el[3] - em[3], m, a);
         mat_dag(a);
         link_at<double>(g, M, y, -em[0], -em[1], -em[2], -em[3], l, c);
-        mat_mul(a, c, t1);
-        link_at<double>(g, L, y, -em[0], -em[1], -em[2], -em[3], m, b);
-        mat_mul(t1, b, t2);
-        mat_axpy(1.0, t2, acc);
-        // U_m(y+l) M_l(y+m) U_m(y)^dag
-        link_at<double>(g, L, y, el[0], el[1], el[2], el[3], m, a);
-        link_at<double>(g, M, y, em[0], em[1], em[2], em[3], l, c);
-        mat_mul(a, c, t1);
-        link_at<double>(g, L, y, 0, 0, 0, 0, m, b);
-        mat_mul_dag(t1, b, t2);
-        mat_axpy(1.0, t2, acc);
+        mat_mul(a, c, t2);
+        link_at<double>(g, M, y, el[0] - em[0], el[1] - em[1], el[2] - em[2], el[3] - em[3], m, c);
+        mat_mul_dag(c, b, t1);
+        mat_axpy(1.0, t1, t2);
+        link_at<double>(g, L, y, -em[0], -em[1], -em[2], -em[3], m, a);
+        mat_mul(t2, a, t1);
+        mat_axpy(1.0, t1, acc);
     }
     mat_axpy(rho, acc, G);
     Mat3<double> U, W;
