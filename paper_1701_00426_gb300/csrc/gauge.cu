@@ -285,6 +285,55 @@ __device__ __forceinline__ void dm_mul(const DM3 &a, const DM3 &b, DM3 &c)
         }
 }
 
+// a <- a b, row by row (a row of the product needs only that row of a), so that
+// no third matrix is live
+__device__ __forceinline__ void mm_inplace(DM3 &a, const DM3 &b)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        DC r[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            Acc2 re, im;
+            acc_zero(re);
+            acc_zero(im);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const DC x = a.e[i * 3 + k], y = b.e[k * 3 + j];
+                acc_prod(re, x.re.x, x.re.y, y.re.x, y.re.y);
+                acc_prod(re, -x.im.x, -x.im.y, y.im.x, y.im.y);
+                acc_prod(im, x.re.x, x.re.y, y.im.x, y.im.y);
+                acc_prod(im, x.im.x, x.im.y, y.re.x, y.re.y);
+            }
+            r[j].re = acc_result(re);
+            r[j].im = acc_result(im);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) a.e[i * 3 + j] = r[j];
+    }
+}
+
+__device__ __forceinline__ void mm_inplace(Mat3<double> &a, const Mat3<double> &b)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        Cplx<double> r[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            double re = 0, im = 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const Cplx<double> x = a.e[i * 3 + k], y = b.e[k * 3 + j];
+                re = fma(x.re, y.re, fma(-x.im, y.im, re));
+                im = fma(x.re, y.im, fma(x.im, y.re, im));
+            }
+            r[j] = {re, im};
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) a.e[i * 3 + j] = r[j];
+    }
+}
+
 // A += s t (s a df64 scalar)
 __device__ __forceinline__ void dm_axpy(float2 s, const DM3 &t, DM3 &A)
 {
@@ -380,6 +429,27 @@ __device__ void staple_sum_df_paths(const LinkGeo &g, const float4 *L, const int
     }
 }
 
+// H -= eps F at one link from M = U A (FP64, about 20 operations): F = traceless
+// part of -(i beta / 6)(M - M^dag), 8 reals with stride Vh.
+__device__ __forceinline__ void gauge_kick(const double (&mre)[9], const double (&mim)[9], double *h, int Vh,
+                                           double beta6, double eps)
+{
+    double f[8];
+    const double d0 = 2.0 * beta6 * mim[0], d1 = 2.0 * beta6 * mim[4], d2 = 2.0 * beta6 * mim[8];
+    const double tr = (d0 + d1 + d2) / 3.0;
+    f[0] = d0 - tr;
+    f[1] = d1 - tr;
+    f[2] = beta6 * (mim[1] + mim[3]);
+    f[3] = beta6 * (mre[3] - mre[1]);
+    f[4] = beta6 * (mim[2] + mim[6]);
+    f[5] = beta6 * (mre[6] - mre[2]);
+    f[6] = beta6 * (mim[5] + mim[7]);
+    f[7] = beta6 * (mre[7] - mre[5]);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) h[(size_t)k * Vh] = fma(-eps, f[k], h[(size_t)k * Vh]);
+}
+
+// The path form, for a device without room for the stored staples.
 // H_mu(x) -= eps F_mu(x) with the staple sum and U A in double-float; F
 // and the update itself in native FP64 (about 20 operations per link).
 __global__ void __launch_bounds__(kGaugeThreads)
@@ -403,20 +473,7 @@ __global__ void __launch_bounds__(kGaugeThreads)
         mre[q] = df_to_f64(M.e[q].re);
         mim[q] = df_to_f64(M.e[q].im);
     }
-    double f[8];
-    const double d0 = 2.0 * beta6 * mim[0], d1 = 2.0 * beta6 * mim[4], d2 = 2.0 * beta6 * mim[8];
-    const double tr = (d0 + d1 + d2) / 3.0;
-    f[0] = d0 - tr;
-    f[1] = d1 - tr;
-    f[2] = beta6 * (mim[1] + mim[3]);
-    f[3] = beta6 * (mre[3] - mre[1]);
-    f[4] = beta6 * (mim[2] + mim[6]);
-    f[5] = beta6 * (mre[6] - mre[2]);
-    f[6] = beta6 * (mim[5] + mim[7]);
-    f[7] = beta6 * (mre[7] - mre[5]);
-    double *h = mom + (size_t)(mp * 8) * Vh + i;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) h[(size_t)k * Vh] = fma(-eps, f[k], h[(size_t)k * Vh]);
+    gauge_kick(mre, mim, mom + (size_t)(mp * 8) * Vh + i, Vh, beta6, eps);
 }
 
 // ------------------------------------------------------------------ scalar arithmetic
@@ -438,6 +495,8 @@ template <class R> __device__ __forceinline__ R r_of(double v);
 template <> __device__ __forceinline__ double r_of<double>(double v) { return v; }
 template <> __device__ __forceinline__ float2 r_of<float2>(double v) { return f64_to_df_slow(v); }
 
+__device__ __forceinline__ double r_double(double a) { return a; }
+__device__ __forceinline__ double r_double(float2 a) { return df_to_f64(a); }
 __device__ __forceinline__ void mm(const Mat3<double> &a, const Mat3<double> &b, Mat3<double> &c) { mat_mul(a, b, c); }
 __device__ __forceinline__ void mm(const DM3 &a, const DM3 &b, DM3 &c) { dm_mul<false>(a, b, c); }
 
@@ -651,6 +710,245 @@ __global__ void __launch_bounds__(kGaugeThreads)
         pn[(size_t)c * Vh] = make_double2(df_to_f64(re), df_to_f64(im));
         pd[(size_t)c * Vh] = make_float4(re.x, re.y, im.x, im.y);
     }
+}
+
+// ------------------------------------------------------------------ force from stored staples
+// The staple sum of the Symanzik action with the plaquette staples as
+// intermediates.  For ordered directions (m, n):
+//   up_mn(x)   = U_n(x) U_m(x+n) U_n(x+m)^dag            (a path from x to x+m)
+//   down_mn(x) = U_n(x-n)^dag U_m(x-n) U_n(x-n+m)
+// and the two sides of a link (mu, x) in the plane of nu, as paths X Y Z from
+// x + mu back to x, carry their three rectangles as one side bent outwards:
+//   c0 X Y Z + c1 (X' Y Z + X Y' Z + X Y Z')
+//     = c1 [ (X Y) (Z' - 20 Z) + (X' Y + X Y') Z ]          5 products
+// (c0 / c1 = -20; c1 goes into the factor beta / 6)
+//   upper: X = U_nu(x+mu), Y = U_mu(x+nu)^dag, Z = U_nu(x)^dag,
+//          X' = up_{nu mu}(x+mu), Y' = up_{mu nu}(x+nu)^dag, Z' = down_{nu mu}(x)^dag
+//   lower: X = U_nu(x+mu-nu)^dag, Y = U_mu(x-nu)^dag, Z = U_nu(x-nu),
+//          X' = up_{nu mu}(x+mu-nu)^dag, Y' = down_{mu nu}(x-nu)^dag, Z' = down_{nu mu}(x-nu)
+// A site's 24 staples cost 36 products (a pair shares its first one), its
+// links' 24 sides 120: 160 products per site with U A, where the separate
+// paths take 340, and 5 neighbour sites per plane instead of 17.  Bound by the
+// FP32 pipes (double-float) or the FP64 pipe (native).  Momentum update,
+// paths -> stored staples: double-float 1542 -> 785 us at 16^4, 7437 -> 3828 at
+// 24^4, 23.2 -> 15.5 ms at 32^4; native 3750 -> 2543 us at 16^4.
+// The staples of np of the six planes at a time are kept (576 bytes per site
+// and plane); the force is linear in A, so planes may be added one pass after
+// another.  Four blocks per SM with two matrices of a thread in shared memory
+// (128 registers); with all in registers (255, two blocks) the update takes
+// 1033 us at 16^4, with three or five blocks 768 and 838 (17.0 and 15.8 ms at
+// 32^4).
+template <class R> struct SideT;
+template <> struct SideT<float2> { using t = float4; };
+template <> struct SideT<double> { using t = double2; };
+
+struct PlaneRange { int p0, np; };
+__device__ __forceinline__ int plane_of(int m, int n)
+{
+    const int a = m < n ? m : n, b = m < n ? n : m;   // 01 02 03 12 13 23
+    return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5);
+}
+// array number of up_mn (down_mn: + 1) among the stored staples
+__device__ __forceinline__ int side_of(const PlaneRange &pr, int m, int n)
+{
+    return ((plane_of(m, n) - pr.p0) * 2 + (m < n ? 0 : 1)) * 2;
+}
+
+struct SiteIdx { int par, idx; };
+__device__ __forceinline__ SiteIdx site_step(const LinkGeo &g, const int (&x)[4], int a, int sa, int b = 0, int sb = 0)
+{
+    int d[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) d[m] = (m == a ? sa : 0) + (m == b ? sb : 0);
+    SiteIdx s;
+    site_of(g, x, d[0], d[1], d[2], d[3], s.par, s.idx);
+    return s;
+}
+
+// Matrix number k of an array of link layout at a site, or its conjugate
+// transpose (read transposed, imaginary parts negated).
+__device__ __forceinline__ void load_side(const float4 *__restrict__ L, int k, SiteIdx s, int Vh, bool dag, DM3 &U)
+{
+    const float4 *p = L + (size_t)((k * 2 + s.par) * 9) * Vh + s.idx;
+    const uint32_t neg = dag ? 0x80000000u : 0u;
+    const size_t row = (size_t)(dag ? 1 : 3) * Vh, col = (size_t)(dag ? 3 : 1) * Vh;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+        const float4 v = __ldg(p + (c / 3) * row + (c % 3) * col);
+        U.e[c].re = make_float2(v.x, v.y);
+        U.e[c].im = xor_sign(make_float2(v.z, v.w), neg);
+    }
+}
+__device__ __forceinline__ void load_side(const double2 *__restrict__ L, int k, SiteIdx s, int Vh, bool dag,
+                                          Mat3<double> &U)
+{
+    const double2 *p = L + (size_t)((k * 2 + s.par) * 9) * Vh + s.idx;
+    const size_t row = (size_t)(dag ? 1 : 3) * Vh, col = (size_t)(dag ? 3 : 1) * Vh;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+        const double2 v = __ldg(p + (c / 3) * row + (c % 3) * col);
+        U.e[c] = {v.x, dag ? -v.y : v.y};
+    }
+}
+__device__ __forceinline__ void store_side(float4 *L, int k, SiteIdx s, int Vh, const DM3 &U)
+{
+    float4 *p = L + (size_t)((k * 2 + s.par) * 9) * Vh + s.idx;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) p[(size_t)c * Vh] = make_float4(U.e[c].re.x, U.e[c].re.y, U.e[c].im.x, U.e[c].im.y);
+}
+__device__ __forceinline__ void store_side(double2 *L, int k, SiteIdx s, int Vh, const Mat3<double> &U)
+{
+    double2 *p = L + (size_t)((k * 2 + s.par) * 9) * Vh + s.idx;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) p[(size_t)c * Vh] = make_double2(U.e[c].re, U.e[c].im);
+}
+
+// a - 20 b
+__device__ __forceinline__ double minus20(double a, double b) { return fma(-20.0, b, a); }
+__device__ __forceinline__ float2 minus20(float2 a, float2 b)
+{
+    float p, e, t, f, h, l;
+    two_prod(-20.f, b.x, p, e);
+    two_sum(a.x, p, t, f);
+    f = __fadd_rn(f, __fadd_rn(a.y, __fmaf_rn(-20.f, b.y, e)));
+    fast_two_sum(t, f, h, l);
+    return make_float2(h, l);
+}
+
+// A thread's matrix in shared memory, [9][kGaugeThreads]: a register matrix
+// less is a block more per SM.
+__device__ __forceinline__ void put_sm(float4 *s, const DM3 &U)
+{
+#pragma unroll
+    for (int c = 0; c < 9; ++c)
+        s[c * kGaugeThreads] = make_float4(U.e[c].re.x, U.e[c].re.y, U.e[c].im.x, U.e[c].im.y);
+}
+__device__ __forceinline__ void put_sm(double2 *s, const Mat3<double> &U)
+{
+#pragma unroll
+    for (int c = 0; c < 9; ++c) s[c * kGaugeThreads] = make_double2(U.e[c].re, U.e[c].im);
+}
+__device__ __forceinline__ Cplx<float2> get_sm(const float4 *s, int c)
+{
+    const float4 v = s[c * kGaugeThreads];
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+}
+__device__ __forceinline__ Cplx<double> get_sm(const double2 *s, int c)
+{
+    const double2 v = s[c * kGaugeThreads];
+    return {v.x, v.y};
+}
+
+// Stored staples of the planes pr: thread = (ordered pair (p, q), parity, site);
+// C = U_p(x) U_q(x+p) gives up_qp(x) = C U_p(x+q)^dag and
+// down_pq(x+q) = U_q(x)^dag C.  One product in a loop: unrolled, the
+// double-float products (about 1300 instructions each) miss the instruction cache.
+template <class R>
+__global__ void __launch_bounds__(kGaugeThreads, 4)
+    k_gauge_sides(LinkGeo g, PlaneRange pr, const typename SideT<R>::t *__restrict__ L, typename SideT<R>::t *__restrict__ F)
+{
+    __shared__ typename SideT<R>::t s_c[9 * kGaugeThreads];
+    const int Vh = g.Vh;
+    const long t = blockIdx.x * (long)kGaugeThreads + threadIdx.x;
+    if (t >= 4L * pr.np * Vh) return;
+    const int i = (int)(t % Vh), w = (int)(t / Vh);
+    const int P = w & 1, pl = pr.p0 + (w >> 2), flip = (w >> 1) & 1;
+    const int a = pl < 3 ? 0 : (pl < 5 ? 1 : 2), b = pl < 3 ? pl + 1 : (pl < 5 ? pl - 1 : 3);
+    const int p = flip ? b : a, q = flip ? a : b;
+    int x[4];
+    coords_of(g, P, i, x);
+    const SiteIdx s0 = {P, i}, sp = site_step(g, x, p, 1), sq = site_step(g, x, q, 1);
+    typename SideT<R>::t *C = s_c + threadIdx.x;
+    Mat3<R> M, u;
+#pragma unroll 1
+    for (int k = 0; k < 3; ++k) {
+        // M u = U_p(x) U_q(x+p) = C; C U_p(x+q)^dag; U_q(x)^dag C
+        if (k != 1) load_side(L, k == 0 ? p : q, s0, Vh, k == 2, M);
+        if (k != 2) load_side(L, k == 0 ? q : p, k == 0 ? sp : sq, Vh, k == 1, u);
+        if (k == 2) {
+#pragma unroll
+            for (int c = 0; c < 9; ++c) u.e[c] = get_sm(C, c);
+        }
+        mm_inplace(M, u);
+        if (k == 0) put_sm(C, M);
+        else store_side(F, k == 1 ? side_of(pr, q, p) : side_of(pr, p, q) + 1, k == 1 ? s0 : sq, Vh, M);
+    }
+}
+
+// H_mu(x) -= eps F of the planes pr from the stored staples (F and the update in
+// FP64).  A block holds the four directions of 32 sites, which share most of
+// the links and staples they read through L1.
+template <class R>
+__global__ void __launch_bounds__(kGaugeThreads, 4)
+    k_gauge_mom_sides(LinkGeo g, PlaneRange pr, const typename SideT<R>::t *__restrict__ L,
+                      const typename SideT<R>::t *__restrict__ F, double *__restrict__ mom, double beta6, double eps)
+{
+    static_assert(kGaugeThreads == 128, "four directions of 32 sites");
+    __shared__ typename SideT<R>::t s_a[9 * kGaugeThreads], s_b[9 * kGaugeThreads];
+    const int Vh = g.Vh, nt = (Vh + 31) / 32;
+    const int P = (int)blockIdx.x / nt, i = ((int)blockIdx.x - P * nt) * 32 + ((int)threadIdx.x & 31);
+    const int mu = (int)threadIdx.x >> 5;
+    if (i >= Vh) return;
+    int x[4];
+    coords_of(g, P, i, x);
+    const SiteIdx s0 = {P, i}, sm = site_step(g, x, mu, 1);
+    typename SideT<R>::t *A = s_a + threadIdx.x, *B = s_b + threadIdx.x;   // sum of the sides; X' Y
+    Mat3<R> M, u;
+    bool any = false;
+#pragma unroll 1
+    for (int w = 0; w < 8; ++w) {
+        const int nu = w >> 1, lower = w & 1;
+        if (nu == mu) continue;
+        const int pl = plane_of(mu, nu);
+        if (pl < pr.p0 || pl >= pr.p0 + pr.np) continue;
+        const SiteIdx sx = lower ? site_step(g, x, mu, 1, nu, -1) : sm;               // X, X'
+        const SiteIdx sy = site_step(g, x, nu, lower ? -1 : 1);                       // Y, Y'
+        const SiteIdx sz = lower ? sy : s0;                                           // Z, Z'
+        const int kx = side_of(pr, nu, mu), ky = side_of(pr, mu, nu) + lower;
+#pragma unroll 1
+        for (int k = 0; k < 5; ++k) {
+            // left factor: X, X Y, X', X, X' Y + X Y'; right: Y, Z' - 20 Z, Y, Y', Z
+            if (k == 0 || k == 2 || k == 3) load_side(k == 2 ? F : L, k == 2 ? kx : nu, sx, Vh, lower != 0, M);
+            const bool zz = k == 1 || k == 4;
+            load_side(k == 3 ? F : L, k == 3 ? ky : (zz ? nu : mu), zz ? sz : sy, Vh, zz ? lower == 0 : true, u);
+            if (k == 1) {
+                Mat3<R> z;
+                load_side(F, kx + 1, sz, Vh, lower == 0, z);
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+                    u.e[q] = {minus20(z.e[q].re, u.e[q].re), minus20(z.e[q].im, u.e[q].im)};
+            }
+            mm_inplace(M, u);
+            if (k == 2) put_sm(B, M);
+            if (k == 3 || k == 4 || k == 1) {
+                // k = 3: M += B; k = 1, 4: A += M
+                if (k == 3 || any) {
+                    const typename SideT<R>::t *y = k == 3 ? B : A;
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) {
+                        const Cplx<R> v = get_sm(y, q);
+                        M.e[q] = {r_add(v.re, M.e[q].re), r_add(v.im, M.e[q].im)};
+                    }
+                }
+                if (k != 3) {
+                    put_sm(A, M);
+                    any = true;
+                }
+            }
+        }
+    }
+    if (!any) return;
+    load_side(L, mu, s0, Vh, false, M);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) u.e[q] = get_sm(A, q);
+    mm_inplace(M, u);
+    double mre[9], mim[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+        mre[q] = r_double(M.e[q].re);
+        mim[q] = r_double(M.e[q].im);
+    }
+    gauge_kick(mre, mim, mom + (size_t)((mu * 2 + P) * 8) * Vh + i, Vh, beta6 * kSymC1, eps);
 }
 
 // IEEE master -> df64 copy (the form k_convert_links writes)
@@ -1522,10 +1820,47 @@ static int check_md(lqcd_ctx *c, int prec)
     return LQCD_OK;
 }
 
+// Planes whose staples are stored at a time: as many of 6, 3, 2, 1 as fit the
+// scratch limit (all six up to 24^4, three at 32^4, one at 48^4: 3.1 GB there).
+// 0: no room even for one plane.
+constexpr size_t kSidesLimit = (size_t)2 << 30;
+
+static int sides_planes(lqcd_ctx *c)
+{
+    const size_t plane = (size_t)1152 * c->Vh;
+    int np = 6;
+    while (np > 1 && np * plane > kSidesLimit) np = np == 6 ? 3 : np - 1;
+    for (; np >= 1; np = np == 6 ? 3 : np - 1) {
+        if (c->md_sides.bytes >= np * plane || c->md_sides.ensure(np * plane) == LQCD_OK) return np;
+        set_error("");
+    }
+    return 0;
+}
+
+template <class R>
+static void launch_mom_sides(lqcd_ctx *c, const typename SideT<R>::t *L, int np, double beta, double eps)
+{
+    const LinkGeo g = link_geo(c);
+    typename SideT<R>::t *F = c->md_sides.as<typename SideT<R>::t>();
+    const unsigned nt = (unsigned)(2 * ((c->Vh + 31) / 32));
+    for (int p0 = 0; p0 < 6; p0 += np) {
+        const PlaneRange pr = {p0, np};
+        k_gauge_sides<R><<<nblocks(4L * np * (long)c->Vh, kGaugeThreads), kGaugeThreads, 0, c->stream>>>(g, pr, L, F);
+        k_gauge_mom_sides<R><<<nt, kGaugeThreads, 0, c->stream>>>(g, pr, L, F, c->mom64.as<double>(), beta / 6.0, eps);
+        c->launches += 2;
+    }
+}
+
 static void launch_mom_update(lqcd_ctx *c, int prec, double beta, double eps)
 {
     const LinkGeo g = link_geo(c);
     const unsigned nb = nblocks(8L * (long)c->Vh, kGaugeThreads);
+    const int np = prec == LQCD_PREC_FP32 ? 0 : sides_planes(c);
+    if (np > 0) {
+        if (prec == LQCD_PREC_FP64) launch_mom_sides<float2>(c, c->lnk_df.as<float4>(), np, beta, eps);
+        else launch_mom_sides<double>(c, c->lnk_nat.as<double2>(), np, beta, eps);
+        return;
+    }
     if (prec == LQCD_PREC_FP64)
         k_gauge_mom_update_df<<<nb, kGaugeThreads, 0, c->stream>>>(g, c->lnk_df.as<float4>(), c->mom64.as<double>(),
                                                                    beta / 6.0, eps);

@@ -152,6 +152,7 @@ struct lqcd_ctx {
     lqcd::DevBuf rat_part;    // per-block partials of its action (+ the total)
     // gauge molecular dynamics (gauge.cu): momenta as 8 reals per link, SoA [4][2][8][Vh]
     lqcd::DevBuf mom64, mom32;
+    lqcd::DevBuf md_sides;    // stored plaquette staples of the FP64 momentum update (gauge.cu)
     lqcd::DevBuf md_part;     // partials of the action / kinetic energy (+ the total)
     lqcd::DevBuf stout_lv;    // stout levels 0 .. n-1 (level 0 = the thin links), IEEE SoA each; level n is lnk_nat
     lqcd::DevBuf stout_M, stout_G;  // force chain scratch: U^dag L and the link's own gradient terms, per link

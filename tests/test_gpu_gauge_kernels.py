@@ -51,3 +51,27 @@ def test_stout_over_sizes_of_rho(gpu, orc, rho, levels):
     grow = max(1.0, 12.0 * rho)
     assert rel(got, orc.stout_smear(dims, U, rho, levels)) <= 1e-13 * grow * levels
     assert rel(force, orc.stout_force(dims, U, rho, F, levels)) <= 1e-12 * (1.0 + 12.0 * rho) ** levels
+
+
+@pytest.mark.parametrize("prec", [0, 3])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 6, 4, 4), (4, 4, 6, 10)])
+@pytest.mark.parametrize("fail", [0, 1])
+def test_momentum_update_from_stored_staples(gpu, orc, prec, dims, fail):
+    """The force from stored plaquette staples against the oracle's paths: wrapping
+    sides of 2, a ragged last block, all six planes at once and (first scratch
+    allocation refused) three at a time.  Bars as for the momentum update:
+    1e-12 double-float, 1e-13 native."""
+    U = inputs.random_links(dims, seed=134)
+    H = inputs.random_momenta(dims, seed=135)
+    eps, beta = 0.03, 5.52
+    ref = orc.mom_update(dims, U, H, beta, eps)
+    with gpu.Context(dims) as c:
+        c.links_upload(U)
+        c.mom_upload(H)
+        gpu.inject_alloc_failure(fail)
+        try:
+            c.gauge_mom_update(beta, eps, prec)
+        finally:
+            gpu.inject_alloc_failure(0)
+        got = c.mom_download()
+    assert rel(got - H, ref - H) <= (1e-12 if prec == 0 else 1e-13)
