@@ -76,7 +76,8 @@ size_t ctx_device_bytes(const lqcd_ctx *c)
                          &c->err_word, &c->io_a, &c->io_b, &c->rat_x, &c->rat_part, &c->mom64,
                          &c->mom32, &c->md_part, &c->ff_y, &c->stout_lv, &c->stout_M, &c->stout_G,
                          &c->stout_F, &c->host_b, &c->host_x, &c->ws.vec, &c->ws.ieee, &c->ws.part, &c->ws.tickets, &c->ws.state,
-                         &c->ws.stage, &c->shard_ws, &c->res_xch, &c->md_sides};
+                         &c->ws.stage, &c->shard_ws, &c->res_xch, &c->md_sides,
+                         &c->mr_vec, &c->mr_ieee, &c->mr_part, &c->mr_tick, &c->mr_st, &c->mr_b, &c->mr_x};
     size_t s = 0;
     for (const DevBuf *p : b) s += p->bytes;
     s += c->ws32.bytes();
@@ -239,7 +240,8 @@ void lqcd_destroy(lqcd_ctx *c)
                    &c->io_a, &c->io_b, &c->rat_x, &c->rat_part, &c->mom64, &c->mom32, &c->md_part, &c->ff_y,
                    &c->stout_lv, &c->stout_M, &c->stout_G, &c->stout_F, &c->host_b, &c->host_x,
                    &c->ws.vec, &c->ws.ieee, &c->ws.part, &c->ws.tickets, &c->ws.state, &c->ws.stage,
-                   &c->shard_ws, &c->res_xch, &c->md_sides};
+                   &c->shard_ws, &c->res_xch, &c->md_sides,
+                   &c->mr_vec, &c->mr_ieee, &c->mr_part, &c->mr_tick, &c->mr_st, &c->mr_b, &c->mr_x};
     for (DevBuf *p : b) p->release();
     c->ws32.release();
     for (Workspace &w : c->ref_ws) w.release();

@@ -2058,7 +2058,7 @@ int lqcd_fermion_force_update(lqcd_ctx *c, double mass, double a0, const double 
     if (!std::isfinite(eps)) return fail(LQCD_EINVAL, "eps is not finite");
     if ((st = links_to_prec(c, LQCD_PREC_FP64_NATIVE)) || (st = mom_to_prec(c, LQCD_PREC_FP64))) return st;
     const size_t n3 = 3 * c->Vh;
-    DevBuf dphi, dr;
+    DevBuf &dphi = c->host_b, &dr = c->host_x;   // kept with the context, as by the host solve
     if ((st = dphi.ensure(n3 * sizeof(double2))) || (st = dr.ensure(n3 * sizeof(double2)))) return st;
     cudaStream_t s = c->stream;
     if ((st = host_to_soa(c, phi, dphi.as<double2>(), 1, s))) return st;

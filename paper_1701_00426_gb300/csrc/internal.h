@@ -160,6 +160,7 @@ struct lqcd_ctx {
     int stout_n = 0;          // active stout levels (0: the links in use are the uploaded ones)
     double stout_rho = 0.0;
     lqcd::DevBuf host_b, host_x;  // device copies of b and x of the host multi-shift call
+    lqcd::DevBuf mr_vec, mr_ieee, mr_part, mr_tick, mr_st, mr_b, mr_x;  // batched CG (mrhs.cu)
     lqcd::DevBuf ff_y;        // D_oe x_i of the fermion force [n][3][Vh] double2
     int md_links_newest = 0;  // LQCD_PREC_FP64: lnk_nat holds the newest links; FP32: lnk_f18
     bool links_derived_stale = false;  // MD moved the links: derived formats need a rebuild
@@ -259,9 +260,11 @@ template <int NJ>
 int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_iter, cudaStream_t s, bool &done);
 
 // helpers shared by solver.cu and mrhs.cu
+uint64_t fnv1a(const void *p, size_t n, uint64_t h = 1469598103934665603ull);   // graph cache keys
 void k_res_nat1_ext(const Geom &g, const double2 *L, const double2 *x, double2 *t, int ntiles, cudaStream_t s);
 void k_res_nat2_ext(const Geom &g, const double2 *L, const double2 *t, const double2 *x, const double2 *b, double a,
                     double2 *r_hi, double *part, unsigned *ticket, double *out, int ntiles, cudaStream_t s);
+void k_norm2_ieee_ext(const double2 *v, int Vh, double *part, unsigned *ticket, int ntiles, double *out, cudaStream_t s);
 double unit_scale_pub(double n2, double n);
 void init_state_pub(SolverState &S, double mass, const double *shifts, int n_shift, double tol_iter, double b2,
                     int max_iter);

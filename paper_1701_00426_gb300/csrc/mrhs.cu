@@ -227,119 +227,176 @@ __global__ void __launch_bounds__(256, R >= 16 ? 1 : 2) k_deo_mrhs_fm(const Mrhs
             A.out[mrhs_at<true>(c, site, j0 + r, Vh, n)] = make_float2(0.5f * acc[r][c].x, 0.5f * acc[r][c].y);
 }
 
-// Per-field deterministic block + tile reduction: vals[r] belongs to field
-// j0 + r of this thread.  fn(j, total) runs once per field in the last block.
-template <int R, class Fn>
-__device__ __forceinline__ void mrhs_reduce(const MrhsArgs &A, const double (&vals)[R], int j0, Fn fn)
+// Fields j0 .. j0 + R - 1 of one colour of a site, 16 bytes (two fields) at a time.
+template <int R>
+__device__ __forceinline__ void mrhs_load(const float2 *p, float2 (&v)[R])
 {
-    __shared__ double s_v[kTile * R];
-    __shared__ int s_last;
+    if constexpr (R % 2 == 0) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) s_v[threadIdx.x * R + r] = vals[r];
+        for (int r = 0; r < R; r += 2) {
+            const float4 t = *reinterpret_cast<const float4 *>(p + r);
+            v[r] = make_float2(t.x, t.y);
+            v[r + 1] = make_float2(t.z, t.w);
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = p[r];
+    }
+}
+template <int R>
+__device__ __forceinline__ void mrhs_store(float2 *p, const float2 (&v)[R])
+{
+    if constexpr (R % 2 == 0) {
+#pragma unroll
+        for (int r = 0; r < R; r += 2)
+            *reinterpret_cast<float4 *>(p + r) = make_float4(v[r].x, v[r].y, v[r + 1].x, v[r + 1].y);
+    } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) p[r] = v[r];
+    }
+}
+
+// Per-field deterministic reduction of a persistent kernel: vals[r] is this
+// thread's sum for field j0 + r over the tiles the block walked.  Lanes of one
+// group meet in a shuffle tree (FP64), the warps in order, and the last block
+// adds the blocks' partials, eight loads at a time, one warp per field; then
+// one warp runs fn(j, total), lane j for field j.  What it costs is paid once
+// per block: with one block per tile (2592 at 24^4, 16 fields) the serial sums
+// of 64 FP64 values and the unbatched sums over the tiles took over half of
+// K3's 72 us (now 31, 0.9 of the copy bandwidth) and 40 of K2's 111 (now 71).
+template <int R, class Fn>
+__device__ __forceinline__ void mrhs_reduce(const MrhsArgs &A, double (&vals)[R], Fn fn)
+{
+    __shared__ double s_v[kTile / 32][kMaxRhs];
+    __shared__ double s_tot[kMaxRhs];
+    __shared__ int s_last;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        for (int o = 16; o >= A.G; o >>= 1) vals[r] += __shfl_xor_sync(0xFFFFFFFFu, vals[r], o);
+    if (lane < A.G) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) s_v[w][lane * R + r] = vals[r];
+    }
     __syncthreads();
-    // field j of this block: threads t with t % G == j / R, slot j % R, in thread order
+    const int nblk = (int)gridDim.x;
     if (threadIdx.x < A.n) {
-        const int j = threadIdx.x, g = j / R, r = j % R;
         double s = 0.0;
-        for (int t = g; t < kTile; t += A.G) s += s_v[t * R + r];
-        A.part[(size_t)j * A.ntiles + blockIdx.x] = s;
+#pragma unroll
+        for (int k = 0; k < kTile / 32; ++k) s += s_v[k][threadIdx.x];
+        A.part[(size_t)threadIdx.x * nblk + blockIdx.x] = s;
+        __threadfence();
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(A.ticket, 1u) == (unsigned)(A.ntiles - 1);
-    }
+    if (threadIdx.x == 0) s_last = atomicAdd(A.ticket, 1u) == (unsigned)(nblk - 1);
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    // one warp per field, lanes strided over tiles, then a fixed shuffle tree
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j = w; j < A.n; j += kTile / 32) {
-        double s = 0.0;
-        for (int k = lane; k < A.ntiles; k += 32) s += __ldcg(A.part + (size_t)j * A.ntiles + k);
+        double s = sum_strided(A.part + (size_t)j * nblk, nblk, lane, 32);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, o);
-        if (lane == 0) fn(j, s);
+        if (lane == 0) s_tot[j] = s;
     }
     __syncthreads();
+    if (threadIdx.x < A.n) fn((int)threadIdx.x, s_tot[threadIdx.x]);
     if (threadIdx.x == 0) *A.ticket = 0u;
 }
 
-// K2: q = a p - D_eo t, <p_j, q_j> per field.
+// K2: q = a p - D_eo t, <p_j, q_j> per field; resident blocks walk the tiles.
 template <int LF, int R>
 __global__ void __launch_bounds__(kTile) k_mrhs_deo2(const MrhsArgs A)
 {
-    const long tid = blockIdx.x * (long)kTile + threadIdx.x;
-    const int site = (int)(tid / A.G);
-    const int grp = (int)(tid - (long)site * A.G);
-    const int j0 = grp * R;
+    const int grp = (int)(threadIdx.x % (unsigned)A.G), j0 = grp * R;   // a tile is a multiple of G threads
     double dots[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) dots[r] = 0.0;
+    float a0[R];
     bool live = false;
 #pragma unroll
-    for (int r = 0; r < R; ++r) live |= A.st[j0 + r].halt == HALT_NONE;
-    if (site < A.g.Vh && live) {
+    for (int r = 0; r < R; ++r) {
+        dots[r] = 0.0;
+        a0[r] = A.st[j0 + r].a0_df.x;
+        live |= A.st[j0 + r].halt == HALT_NONE;
+    }
+    for (int tile = blockIdx.x; live && tile < A.ntiles; tile += gridDim.x) {
+        const int site = (int)(((long)tile * kTile + threadIdx.x) / A.G);
+        if (site >= A.g.Vh) break;
         Stencil S;
         make_stencil(A.g, site, 0, S);
         float2 acc[R][3];
         mrhs_site<LF, R>(A, S, site, j0, acc);
+        float d[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const SolverState *st = A.st + j0 + r;
-            const float a = st->a0_df.x;
-            float d = 0.f;
+        for (int r = 0; r < R; ++r) d[r] = 0.f;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0 + r;
-                const float2 pv = A.p[o];
-                const float2 qv = make_float2(__fmaf_rn(a, pv.x, -0.5f * acc[r][c].x), __fmaf_rn(a, pv.y, -0.5f * acc[r][c].y));
-                A.out[o] = qv;
-                d = __fmaf_rn(pv.x, qv.x, __fmaf_rn(pv.y, qv.y, d));
+        for (int c = 0; c < 3; ++c) {
+            const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0;
+            float2 pv[R], qv[R];
+            mrhs_load<R>(A.p + o, pv);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                qv[r] = make_float2(__fmaf_rn(a0[r], pv[r].x, -0.5f * acc[r][c].x),
+                                    __fmaf_rn(a0[r], pv[r].y, -0.5f * acc[r][c].y));
+                d[r] = __fmaf_rn(pv[r].x, qv[r].x, __fmaf_rn(pv[r].y, qv[r].y, d[r]));
             }
-            dots[r] = (double)d;
+            mrhs_store<R>(A.out + o, qv);
         }
+#pragma unroll
+        for (int r = 0; r < R; ++r) dots[r] += (double)d[r];
     }
-    mrhs_reduce<R>(A, dots, j0, [&](int j, double tot) {
+    mrhs_reduce<R>(A, dots, [&](int j, double tot) {
         if (!A.st[j].halt) finalize_pq(A.st + j, tot);
     });
 }
 
-// K3: r -= alpha_j q, ||r_j||^2 (in = q, out = r)
+// K3: r -= alpha_j q, ||r_j||^2 (in = q, out = r); a stopped field keeps its r.
 template <int R>
 __global__ void __launch_bounds__(kTile) k_mrhs_upd_r(const MrhsArgs A)
 {
-    const long tid = blockIdx.x * (long)kTile + threadIdx.x;
-    const int site = (int)(tid / A.G);
-    const int grp = (int)(tid - (long)site * A.G);
-    const int j0 = grp * R;
+    const int grp = (int)(threadIdx.x % (unsigned)A.G), j0 = grp * R;
     double nr[R];
+    float na[R];
+    bool on[R], any = false;
 #pragma unroll
-    for (int r = 0; r < R; ++r) nr[r] = 0.0;
-    if (site < A.g.Vh) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const SolverState *st = A.st + j0 + r;
-            if (st->halt) continue;
-            const float na = -st->alpha_df.x;
-            float d = 0.f;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0 + r;
-                const float2 qv = A.in[o], rv = A.out[o];
-                const float2 w = make_float2(__fmaf_rn(na, qv.x, rv.x), __fmaf_rn(na, qv.y, rv.y));
-                A.out[o] = w;
-                d = __fmaf_rn(w.x, w.x, __fmaf_rn(w.y, w.y, d));
-            }
-            nr[r] = (double)d;
-        }
+    for (int r = 0; r < R; ++r) {
+        nr[r] = 0.0;
+        na[r] = -A.st[j0 + r].alpha_df.x;
+        on[r] = A.st[j0 + r].halt == HALT_NONE;
+        any |= on[r];
     }
-    mrhs_reduce<R>(A, nr, j0, [&](int j, double tot) {
+    for (int tile = blockIdx.x; any && tile < A.ntiles; tile += gridDim.x) {
+        const int site = (int)(((long)tile * kTile + threadIdx.x) / A.G);
+        if (site >= A.g.Vh) break;
+        float2 qv[3][R], rv[3][R];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0;
+            mrhs_load<R>(A.in + o, qv[c]);
+            mrhs_load<R>(A.out + o, rv[c]);
+        }
+        float d[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) d[r] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float2 x = make_float2(__fmaf_rn(na[r], qv[c][r].x, rv[c][r].x),
+                                             __fmaf_rn(na[r], qv[c][r].y, rv[c][r].y));
+                if (on[r]) rv[c][r] = x;
+                d[r] = __fmaf_rn(x.x, x.x, __fmaf_rn(x.y, x.y, d[r]));
+            }
+            mrhs_store<R>(A.out + ((size_t)c * A.g.Vh + site) * A.n + j0, rv[c]);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) nr[r] += (double)d[r];
+    }
+    mrhs_reduce<R>(A, nr, [&](int j, double tot) {
         if (!A.st[j].halt) finalize_rr(A.st + j, tot);
     });
 }
 
-// K4: x_j += alpha_j p_j; p_j = r_j + beta_j p_j (in = r, out = x, p = p)
+// K4: x_j += alpha_j p_j; p_j = r_j + beta_j p_j (in = r, out = x, p = p).  HBM
+// bound; two fields per access instead of one: 70 -> 36 us at 24^4, 16 fields.
 template <int R>
 __global__ void __launch_bounds__(kTile) k_mrhs_upd_xp(const MrhsArgs A, float2 *pvec)
 {
@@ -348,18 +405,37 @@ __global__ void __launch_bounds__(kTile) k_mrhs_upd_xp(const MrhsArgs A, float2 
     const int grp = (int)(tid - (long)site * A.G);
     if (site >= A.g.Vh) return;
     const int j0 = grp * R;
+    float as[R], bs[R];
+    bool on[R], any = false;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const SolverState *st = A.st + j0 + r;
-        if (!st->do_k4) continue;
-        const float as = st->alpha_s_df[0].x, bs = st->beta_s_df[0].x;
+        on[r] = st->do_k4 != 0;
+        any |= on[r];
+        as[r] = st->alpha_s_df[0].x;
+        bs[r] = st->beta_s_df[0].x;
+    }
+    if (!any) return;
+    float2 pv[3][R], xv[3][R], rv[3][R];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0 + r;
-            const float2 pv = pvec[o], xv = A.out[o], rv = A.in[o];
-            A.out[o] = make_float2(__fmaf_rn(as, pv.x, xv.x), __fmaf_rn(as, pv.y, xv.y));
-            pvec[o] = make_float2(__fmaf_rn(bs, pv.x, rv.x), __fmaf_rn(bs, pv.y, rv.y));
+    for (int c = 0; c < 3; ++c) {
+        const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0;
+        mrhs_load<R>(pvec + o, pv[c]);
+        mrhs_load<R>(A.out + o, xv[c]);
+        mrhs_load<R>(A.in + o, rv[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const size_t o = ((size_t)c * A.g.Vh + site) * A.n + j0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (!on[r]) continue;   // a stopped field keeps its x and p
+            const float2 p = pv[c][r];
+            xv[c][r] = make_float2(__fmaf_rn(as[r], p.x, xv[c][r].x), __fmaf_rn(as[r], p.y, xv[c][r].y));
+            pv[c][r] = make_float2(__fmaf_rn(bs[r], p.x, rv[c][r].x), __fmaf_rn(bs[r], p.y, rv[c][r].y));
         }
+        mrhs_store<R>(A.out + o, xv[c]);
+        mrhs_store<R>(pvec + o, pv[c]);
     }
 }
 
@@ -444,6 +520,35 @@ static void launch_deo2_R(const MrhsArgs &A, int R, unsigned nb, cudaStream_t s)
     if (R == 4) k_mrhs_deo2<LF, 4><<<nb, kTile, 0, s>>>(A);
     else if (R == 2) k_mrhs_deo2<LF, 2><<<nb, kTile, 0, s>>>(A);
     else k_mrhs_deo2<LF, 1><<<nb, kTile, 0, s>>>(A);
+}
+
+static void launch_deo2(const MrhsArgs &A, int lf, int R, unsigned nb, cudaStream_t s)
+{
+    if (lf == LF_F32_18) launch_deo2_R<LF_F32_18>(A, R, nb, s);
+    else if (lf == LF_F32_12) launch_deo2_R<LF_F32_12>(A, R, nb, s);
+    else launch_deo2_R<LF_F16_12>(A, R, nb, s);
+}
+
+// Blocks of kern that fit on the current device at once.
+template <class K>
+static unsigned resident_grid(K kern, int ntiles)
+{
+    int dev = 0, nsm = 0, occ = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kTile, 0) != cudaSuccess || occ < 1) {
+        cudaGetLastError();
+        return (unsigned)ntiles;
+    }
+    return (unsigned)std::min(ntiles, occ * nsm);
+}
+
+template <int R>
+static unsigned deo2_grid(int lf, int ntiles)
+{
+    if (lf == LF_F32_18) return resident_grid(k_mrhs_deo2<LF_F32_18, R>, ntiles);
+    if (lf == LF_F32_12) return resident_grid(k_mrhs_deo2<LF_F32_12, R>, ntiles);
+    return resident_grid(k_mrhs_deo2<LF_F16_12, R>, ntiles);
 }
 
 // Fields per thread of the stand-alone multi-RHS D_eo, picked per (n, recon,
@@ -533,8 +638,8 @@ int deo_mrhs_launch(lqcd_ctx *c, int P, int n, int recon, const void *in, void *
 // Batched CG core on the device.  n fields (1..16, padded internally to a
 // power of two so that the fields of a site never straddle a block), field j
 // solves (A + sigma[j]) x_j = b_j with b_j = b + j * b_stride * 3 Vh (stride 0:
-// one shared source), starting from the IEEE guess in xh[j] and leaving the
-// FP64 solution there.  lf: link storage of the FP32 iterations.
+// one shared source); xh[j] is zero on entry and holds the FP64 solution
+// afterwards.  lf: link storage of the FP32 iterations.
 // infos[j] (may be NULL) receive iterations, reliable updates and the FP64
 // true residual; bytes accumulates the algorithmic traffic.
 int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double tol, const double2 *b,
@@ -548,44 +653,56 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
     const int R = np >= 4 ? 4 : np, G = np / R;
     const int ntiles = (int)((Vh * G + kTile - 1) / kTile);
     const void *links = lf == LF_F16_12 ? c->lnk_h12.ptr : (lf == LF_F32_12 ? c->lnk_f12.ptr : c->lnk_f18.ptr);
-    DevBuf vec, ieee, part, tick, stb;
+    // the workspace stays with the context (grown, never shrunk): repeated
+    // calls allocate nothing
+    DevBuf &vec = c->mr_vec, &ieee = c->mr_ieee, &part = c->mr_part, &tick = c->mr_tick, &stb = c->mr_st;
     int st;
+    const unsigned nb = (unsigned)ntiles;
+    const unsigned nb2 = R == 4 ? deo2_grid<4>(lf, ntiles) : (R == 2 ? deo2_grid<2>(lf, ntiles) : deo2_grid<1>(lf, ntiles));
+    const unsigned nbr = R == 4 ? resident_grid(k_mrhs_upd_r<4>, ntiles)
+                                : (R == 2 ? resident_grid(k_mrhs_upd_r<2>, ntiles) : resident_grid(k_mrhs_upd_r<1>, ntiles));
+    const int nt1 = (int)((Vh + kTile - 1) / kTile);
+    const size_t npart = std::max((size_t)np * std::max(nb2, nbr), (size_t)nt1);
     if ((st = vec.ensure(5 * (size_t)n3 * np * sizeof(float2)))) return st;
-    if ((st = ieee.ensure(2 * (size_t)n3 * sizeof(double2)))) return st;
-    if ((st = part.ensure(((size_t)np * ntiles + 64) * sizeof(double)))) return st;
+    if ((st = ieee.ensure((size_t)(n + 1) * n3 * sizeof(double2)))) return st;
+    if ((st = part.ensure((npart + 64) * sizeof(double)))) return st;
     if ((st = tick.ensure(64))) return st;
     if ((st = stb.ensure((size_t)np * sizeof(SolverState)))) return st;
     LQCD_CUDA(cudaMemsetAsync(tick.ptr, 0, 64, s));
     LQCD_CUDA(cudaMemsetAsync(vec.ptr, 0, 5 * (size_t)n3 * np * sizeof(float2), s));
     float2 *r = vec.as<float2>(), *p = r + n3 * np, *x = p + n3 * np, *q = x + n3 * np, *t = q + n3 * np;
-    double2 *rh = ieee.as<double2>(), *tn = rh + n3;
+    double2 *rh = ieee.as<double2>(), *tn = rh + (size_t)n * n3;   // residuals of all fields, one temporary
     SolverState *sts = stb.as<SolverState>();
-    double *partd = part.as<double>(), *res = partd + (size_t)np * ntiles;
+    double *partd = part.as<double>(), *res = partd + npart;
     unsigned *tk = tick.as<unsigned>();
     const double2 *Lnat = c->lnk_nat.as<double2>();
-    const int nt1 = (int)((Vh + kTile - 1) / kTile);
     const unsigned nb3 = (unsigned)((n3 + 255) / 256);
     auto bj = [&](int j) { return b + (size_t)j * b_stride * n3; };
-    auto true_res = [&](int j, double &rr) -> int {
-        const double a = mass * mass + sigma[j];
-        k_res_nat1_ext(c->g, Lnat, xh + (size_t)j * n3, tn, nt1, s);
-        k_res_nat2_ext(c->g, Lnat, tn, xh + (size_t)j * n3, bj(j), a, rh, partd, tk + 1, res, nt1, s);
-        LQCD_CUDA(cudaGetLastError());
-        c->launches += 2;
-        LQCD_CUDA(cudaMemcpyAsync(c->h_pinned_d, res, sizeof(double), cudaMemcpyDeviceToHost, s));
+    // FP64 true residuals of the fields listed, into rh and rr: all launches, then
+    // one synchronisation
+    auto true_res = [&](const std::vector<int> &js, std::vector<double> &rr) -> int {
+        for (int j : js) {
+            const double a = mass * mass + sigma[j];
+            k_res_nat1_ext(c->g, Lnat, xh + (size_t)j * n3, tn, nt1, s);
+            k_res_nat2_ext(c->g, Lnat, tn, xh + (size_t)j * n3, bj(j), a, rh + (size_t)j * n3, partd, tk + 1, res + j, nt1,
+                           s);
+            LQCD_CUDA(cudaGetLastError());
+            c->launches += 2;
+        }
+        LQCD_CUDA(cudaMemcpyAsync(c->h_pinned_d, res, kMaxRhs * sizeof(double), cudaMemcpyDeviceToHost, s));
         LQCD_CUDA(cudaStreamSynchronize(s));
-        rr = c->h_pinned_d[0];
+        for (int j : js) rr[j] = c->h_pinned_d[j];
         return LQCD_OK;
     };
-    std::vector<double> b2(np, 0.0), scale(np, 1.0), target2(np, 0.0);
+    std::vector<double> b2(np, 0.0), scale(np, 1.0), target2(np, 0.0), rr(np, 0.0);
     std::vector<int> done(np, 1), rel(np, 0);
     const double delta = c->opts.delta_reliable;
     // (re)start field j from the IEEE residual in rh: FP32 residual scaled to
     // O(1) entries, x_lo = 0, p kept (rescaled) or set to r
-    auto restart = [&](int j, double rr, const SolverState *prev) -> int {
+    auto restart = [&](int j, const SolverState *prev) -> int {
         const double old = scale[j];
-        scale[j] = unit_scale_pub(rr, 6.0 * Vh);
-        k_col_from_ieee<<<nb3, 256, 0, s>>>(rh, r, n3, np, j, scale[j]);
+        scale[j] = unit_scale_pub(rr[j], 6.0 * Vh);
+        k_col_from_ieee<<<nb3, 256, 0, s>>>(rh + (size_t)j * n3, r, n3, np, j, scale[j]);
         k_col_set<<<nb3, 256, 0, s>>>(x, nullptr, n3, np, j, 1);
         if (prev)
             k_col_scale<<<nb3, 256, 0, s>>>(p, n3, np, j, (float)(scale[j] / old));
@@ -593,7 +710,7 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
             k_col_set<<<nb3, 256, 0, s>>>(p, r, n3, np, j, 0);
         LQCD_CUDA(cudaGetLastError());
         c->launches += 3;
-        const double rho = rr * scale[j] * scale[j];
+        const double rho = rr[j] * scale[j] * scale[j];
         SolverState T;
         if (prev) {
             T = *prev;
@@ -612,29 +729,24 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
     memset(&idle, 0, sizeof idle);
     idle.halt = HALT_CONVERGED;
     for (int j = 0; j < np; ++j) LQCD_CUDA(cudaMemcpyAsync(sts + j, &idle, sizeof idle, cudaMemcpyHostToDevice, s));
+    // ||b_j||^2; the guess is zero, so b_j is also the first residual
+    std::vector<int> all_j(n);
     for (int j = 0; j < n; ++j) {
-        LQCD_CUDA(cudaMemsetAsync(tn, 0, n3 * sizeof(double2), s));
-        // ||b_j||^2 from the residual of x = 0 (A applied to zero)
-        double2 *xj = xh + (size_t)j * n3;
-        {
-            const double a = mass * mass + sigma[j];
-            k_res_nat2_ext(c->g, Lnat, tn, tn, bj(j), a, nullptr, partd, tk + 1, res, nt1, s);
-            LQCD_CUDA(cudaGetLastError());
-            LQCD_CUDA(cudaMemcpyAsync(c->h_pinned_d, res, sizeof(double), cudaMemcpyDeviceToHost, s));
-            LQCD_CUDA(cudaStreamSynchronize(s));
-            b2[j] = c->h_pinned_d[0];
-        }
+        all_j[j] = j;
+        k_norm2_ieee_ext(bj(j), (int)Vh, partd, tk + 1, nt1, res + j, s);
+        LQCD_CUDA(cudaMemcpyAsync(rh + (size_t)j * n3, bj(j), n3 * sizeof(double2), cudaMemcpyDeviceToDevice, s));
+    }
+    LQCD_CUDA(cudaGetLastError());
+    c->launches += n;
+    LQCD_CUDA(cudaMemcpyAsync(c->h_pinned_d, res, kMaxRhs * sizeof(double), cudaMemcpyDeviceToHost, s));
+    LQCD_CUDA(cudaStreamSynchronize(s));
+    for (int j = 0; j < n; ++j) {
+        b2[j] = rr[j] = c->h_pinned_d[j];
         if (!std::isfinite(b2[j])) return fail(LQCD_ENAN, "source contains NaN/Inf");
         target2[j] = tol * tol * b2[j];
-        if (b2[j] == 0.0) {
-            LQCD_CUDA(cudaMemsetAsync(xj, 0, n3 * sizeof(double2), s));
-            continue;
-        }
-        double rr;
-        if ((st = true_res(j, rr))) return st;
-        if (rr <= target2[j]) continue;
+        if (rr[j] <= target2[j]) continue;   // b_j = 0, or tol >= 1: x_j = 0
         done[j] = 0;
-        if ((st = restart(j, rr, nullptr))) return st;
+        if ((st = restart(j, nullptr))) return st;
     }
     MrhsArgs A;
     memset(&A, 0, sizeof A);
@@ -646,31 +758,34 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
     A.part = partd;
     A.ticket = tk;
     A.ntiles = ntiles;
-    const unsigned nb = (unsigned)ntiles;
     MrhsArgs A1 = A, A2 = A, A3 = A, A4 = A;
     A1.P = 1; A1.in = p; A1.out = t;
     A2.P = 0; A2.in = t; A2.out = q; A2.p = p;
     A3.in = q; A3.out = r;
     A4.in = r; A4.out = x;
     const int chunk = c->opts.check_every;
-    cudaGraphExec_t exec = nullptr;
-    {
+    // the chunk's graph is kept with the context: the scalars are on the device,
+    // so it depends on the workspace and the launch shapes only
+    const unsigned shape[5] = {nb, nb2, nbr, (unsigned)lf, (unsigned)chunk};
+    uint64_t key = fnv1a(&A1, sizeof A1, fnv1a(&A2, sizeof A2, fnv1a(&A3, sizeof A3, fnv1a(&A4, sizeof A4))));
+    key = fnv1a(shape, sizeof shape, key);
+    cudaGraphExec_t exec = c->graph.find(key);
+    if (!exec) {
         cudaGraph_t g;
         LQCD_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
         for (int k = 0; k < chunk; ++k) {
             launch_deo_mrhs(A1, lf, R, nb, s);
-            if (lf == LF_F32_18) launch_deo2_R<LF_F32_18>(A2, R, nb, s);
-            else if (lf == LF_F32_12) launch_deo2_R<LF_F32_12>(A2, R, nb, s);
-            else launch_deo2_R<LF_F16_12>(A2, R, nb, s);
-            if (R == 4) { k_mrhs_upd_r<4><<<nb, kTile, 0, s>>>(A3); k_mrhs_upd_xp<4><<<nb, kTile, 0, s>>>(A4, p); }
-            else if (R == 2) { k_mrhs_upd_r<2><<<nb, kTile, 0, s>>>(A3); k_mrhs_upd_xp<2><<<nb, kTile, 0, s>>>(A4, p); }
-            else { k_mrhs_upd_r<1><<<nb, kTile, 0, s>>>(A3); k_mrhs_upd_xp<1><<<nb, kTile, 0, s>>>(A4, p); }
+            launch_deo2(A2, lf, R, nb2, s);
+            if (R == 4) { k_mrhs_upd_r<4><<<nbr, kTile, 0, s>>>(A3); k_mrhs_upd_xp<4><<<nb, kTile, 0, s>>>(A4, p); }
+            else if (R == 2) { k_mrhs_upd_r<2><<<nbr, kTile, 0, s>>>(A3); k_mrhs_upd_xp<2><<<nb, kTile, 0, s>>>(A4, p); }
+            else { k_mrhs_upd_r<1><<<nbr, kTile, 0, s>>>(A3); k_mrhs_upd_xp<1><<<nb, kTile, 0, s>>>(A4, p); }
         }
         cudaError_t e = cudaStreamEndCapture(s, &g);
         if (e != cudaSuccess) return cuda_fail(e, "batched CG graph capture");
         e = cudaGraphInstantiate(&exec, g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return cuda_fail(e, "batched CG graph instantiate");
+        c->graph.put(key, exec);
     }
     int *hs = c->h_pinned;
     std::vector<SolverState> O(np);
@@ -701,19 +816,22 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
         if (rc) break;
         cudaError_t e = cudaMemcpy(O.data(), sts, (size_t)np * sizeof(SolverState), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) { rc = cuda_fail(e, "batched CG state"); break; }
-        bool progressed = false;
+        // the fields that stopped: solution updated, FP64 residual, next segment
+        std::vector<int> js;
         for (int j = 0; j < n && rc == LQCD_OK; ++j) {
             if (done[j] || O[j].halt == HALT_NONE) continue;
-            progressed = true;
             iters[j] = O[j].iters;
             if (O[j].halt == HALT_NAN) { rc = fail(LQCD_ENAN, "NaN/Inf or breakdown in the batched CG"); break; }
             k_col_to_ieee_add<<<nb3, 256, 0, s>>>(x, xh + (size_t)j * n3, n3, np, j, 1.0 / scale[j]);
             c->launches += 1;
-            double rr;
-            if ((rc = true_res(j, rr))) break;
+            js.push_back(j);
+        }
+        if (rc == LQCD_OK && !js.empty()) rc = true_res(js, rr);
+        for (size_t k = 0; k < js.size() && rc == LQCD_OK; ++k) {
+            const int j = js[k];
             if (O[j].halt == HALT_MAXITER) { done[j] = 2; continue; }
             if (O[j].halt == HALT_RELIABLE) ++rel[j];
-            if (rr <= target2[j]) {
+            if (rr[j] <= target2[j]) {
                 done[j] = 1;
                 SolverState T = O[j];
                 T.halt = HALT_CONVERGED;
@@ -721,19 +839,22 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
                 if (e != cudaSuccess) rc = cuda_fail(e, "batched CG state");
                 continue;
             }
-            rc = restart(j, rr, &O[j]);
+            rc = restart(j, &O[j]);
         }
-        if (!progressed && rc == LQCD_OK)
+        if (js.empty() && rc == LQCD_OK)
             for (int j = 0; j < n; ++j)
                 if (!done[j]) done[j] = 2;
     }
-    cudaGraphExecDestroy(exec);
     if (rc) return rc;
+    // rr[j] is the residual of the x_j returned, but for a field whose iteration
+    // was given up without a halt
+    std::vector<int> open;
+    for (int j = 0; j < n; ++j)
+        if (done[j] == 2) open.push_back(j);
+    if (!open.empty() && (st = true_res(open, rr))) return st;
     int status = LQCD_OK;
     for (int j = 0; j < n; ++j) {
-        double rr = 0;
-        if (b2[j] > 0 && (st = true_res(j, rr))) return st;
-        const double res_j = b2[j] > 0 ? std::sqrt(rr / b2[j]) : 0.0;
+        const double res_j = b2[j] > 0 ? std::sqrt(rr[j] / b2[j]) : 0.0;
         if (!(res_j <= tol)) status = LQCD_ENOCONV;
         if (infos) {
             lqcd_solve_info &I = infos[j];
@@ -760,7 +881,7 @@ int cg_solve_mrhs(lqcd_ctx *c, double mass, double sigma, int n, double tol, con
         return fail(LQCD_EINVAL, "need tol > 0, sigma >= 0 and m^2 + sigma > 0");
     cudaStream_t s = c->stream;
     const size_t n3 = 3 * c->Vh;
-    DevBuf bd, xd;
+    DevBuf &bd = c->mr_b, &xd = c->mr_x;
     int st;
     if ((st = bd.ensure((size_t)n * n3 * sizeof(double2))) || (st = xd.ensure((size_t)n * n3 * sizeof(double2))))
         return st;

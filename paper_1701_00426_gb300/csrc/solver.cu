@@ -255,6 +255,11 @@ void k_res_nat2_ext(const Geom &g, const double2 *L, const double2 *t, const dou
     k_res_nat2<VP_F32><<<ntiles, kTile, 0, s>>>(g, L, t, x, b, a, r_hi, nullptr, 1.0, part, ticket, out);
 }
 
+void k_norm2_ieee_ext(const double2 *v, int Vh, double *part, unsigned *ticket, int ntiles, double *out, cudaStream_t s)
+{
+    k_norm2_ieee<<<ntiles, kTile, 0, s>>>(v, Vh, 1, part, ticket, ntiles, out);
+}
+
 // ------------------------------------------------------------------ workspace
 
 
@@ -571,7 +576,7 @@ void GraphCache::put(uint64_t k, cudaGraphExec_t g)
     used[v] = ++tick;
 }
 
-static uint64_t fnv1a(const void *p, size_t n, uint64_t h = 1469598103934665603ull)
+uint64_t fnv1a(const void *p, size_t n, uint64_t h)
 {
     const unsigned char *b = (const unsigned char *)p;
     for (size_t i = 0; i < n; ++i) {
@@ -1374,7 +1379,6 @@ int mscg_solve_packed(lqcd_ctx *const *ctxs, int n, const double *mass, const do
     lqcd_ctx *c0 = ctxs[0];
     cudaStream_t s = c0->stream;
     std::vector<JobRun> J(n);
-    std::vector<DevBuf> bd(n), xd(n);
     int st;
     for (int i = 0; i < n; ++i) {
         lqcd_ctx *c = ctxs[i];
@@ -1383,15 +1387,17 @@ int mscg_solve_packed(lqcd_ctx *const *ctxs, int n, const double *mass, const do
         for (int k = 0; k < i; ++k)
             if (ctxs[k] == c) return fail(LQCD_EINVAL, "a context appears twice in a packed solve");
         const size_t n3 = 3 * c->Vh;
-        if ((st = bd[i].ensure(n3 * sizeof(double2))) || (st = xd[i].ensure((size_t)n_shift[i] * n3 * sizeof(double2))))
+        // device copies of b and x: those of the context's host call (kept)
+        if ((st = c->host_b.ensure(n3 * sizeof(double2))) ||
+            (st = c->host_x.ensure((size_t)n_shift[i] * n3 * sizeof(double2))))
             return st;
-        if ((st = job_init(J[i], c, nullptr, mass[i], shifts[i], n_shift[i], tol[i], bd[i].as<double2>(),
-                           xd[i].as<double2>())))
+        if ((st = job_init(J[i], c, nullptr, mass[i], shifts[i], n_shift[i], tol[i], c->host_b.as<double2>(),
+                           c->host_x.as<double2>())))
             return st;
         if (i > 0 && J[i].vp != J[0].vp) return fail(LQCD_EINVAL, "packed contexts must use the same precision");
         if (i > 0 && J[i].lf != J[0].lf) return fail(LQCD_EINVAL, "packed contexts must use the same link storage");
         LQCD_CUDA(cudaStreamSynchronize(c->stream));
-        if ((st = host_to_soa(c, b[i], bd[i].as<double2>(), 1, s))) return st;
+        if ((st = host_to_soa(c, b[i], c->host_b.as<double2>(), 1, s))) return st;
         if ((st = job_setup(J[i], s))) return st;
     }
     IterBatch<kMaxJobs> B;
@@ -1414,7 +1420,7 @@ int mscg_solve_packed(lqcd_ctx *const *ctxs, int n, const double *mass, const do
         st = job_finish(J[i], s);
         if (st != LQCD_OK && st != LQCD_ENOCONV) return st;
         if (st == LQCD_ENOCONV) status = st;
-        if ((st = soa_to_host(ctxs[i], xd[i].as<double2>(), x[i], n_shift[i], s))) return st;
+        if ((st = soa_to_host(ctxs[i], ctxs[i]->host_x.as<double2>(), x[i], n_shift[i], s))) return st;
         LQCD_CUDA(cudaStreamSynchronize(s));
         J[i].I.secs = secs_iter;
         if (info) info[i] = J[i].I;
