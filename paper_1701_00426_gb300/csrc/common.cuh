@@ -426,6 +426,18 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy()
 #endif
 }
 
+// The normal priority as a policy, for links that are read again from L2.
+__device__ __forceinline__ uint64_t l2_normal_policy()
+{
+#ifdef LQCD_NO_L2_HINTS
+    return 0;
+#else
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
+#endif
+}
+
 __device__ __forceinline__ float4 ldg4_stream(const float4 *p, uint64_t pol)
 {
 #ifdef LQCD_NO_L2_HINTS

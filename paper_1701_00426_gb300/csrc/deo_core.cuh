@@ -286,11 +286,11 @@ __device__ __forceinline__ float2 h2f(uint32_t w)
 }
 
 // Links are streamed once per application: loads carry the L2 evict-first
-// policy so that the re-read spinors keep their place in L2.
+// policy so that the re-read spinors keep their place in L2 (pol: another one).
 template <int LF>
-__device__ __forceinline__ void load_link_f32(const void *L, int mu, int par, int idx, int Vh, float2 (&U)[9])
+__device__ __forceinline__ void load_link_f32(const void *L, int mu, int par, int idx, int Vh, float2 (&U)[9],
+                                              uint64_t pol = l2_evict_first_policy())
 {
-    const uint64_t pol = l2_evict_first_policy();
     if (LF == LF_F32_18) {
         const float2 *p = (const float2 *)L + link_base(mu, par, 9, Vh) + idx;
 #pragma unroll
@@ -321,7 +321,8 @@ __device__ __forceinline__ void load_link_f32(const void *L, int mu, int par, in
 // order are the same, so are the bits.
 template <int LF, int UNROLL = 1>
 __device__ __forceinline__ void deo_site_f32(const Geom &g, const void *L, const float2 *in, const Stencil &S, int i,
-                                             int P, int Vh, float2 (&res)[3])
+                                             int P, int Vh, float2 (&res)[3],
+                                             uint64_t pol = l2_evict_first_policy())
 {
     float2 acc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll UNROLL
@@ -330,7 +331,7 @@ __device__ __forceinline__ void deo_site_f32(const Geom &g, const void *L, const
         uint32_t nf, nb;
         hop(g, S, mu, f, b, nf, nb);
         float2 U[9], v[3];
-        load_link_f32<LF>(L, mu, P, i, Vh, U);
+        load_link_f32<LF>(L, mu, P, i, Vh, U, pol);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float2 t = ldg2(in + (size_t)c * Vh + f);
@@ -345,7 +346,7 @@ __device__ __forceinline__ void deo_site_f32(const Geom &g, const void *L, const
                 acc[a].x = __fmaf_rn(u.x, v[b].x, __fmaf_rn(-u.y, v[b].y, acc[a].x));
                 acc[a].y = __fmaf_rn(u.x, v[b].y, __fmaf_rn(u.y, v[b].x, acc[a].y));
             }
-        load_link_f32<LF>(L, mu, 1 - P, b, Vh, U);
+        load_link_f32<LF>(L, mu, 1 - P, b, Vh, U, pol);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const float2 t = ldg2(in + (size_t)c * Vh + b);

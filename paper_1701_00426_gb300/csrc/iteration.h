@@ -50,6 +50,7 @@ struct IterJob {
     double *part;        // per-tile partial sums
     unsigned *ticket;    // last-block-done counter
     int tile0, ntiles;
+    int keep;            // FP32 / FP16 links stay in L2 between the stencils: normal priority instead of evict-first
 };
 
 template <int NJ>

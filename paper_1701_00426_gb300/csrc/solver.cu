@@ -415,11 +415,11 @@ static int staged_solver_blocks()
     return g_st_blocks[dev];
 }
 
-// Grid of the persistent reduction kernels (FP32 / FP16 K2, K3 of every
+// Grids of the persistent reduction kernels (FP32 / FP16 K2, K3 of every
 // precision): the resident blocks of the FP32 K2 (all link formats and batch
-// sizes), once per device; 0 = the one-block-per-tile k_it_deo2 /
+// sizes) and of K3, once per device; 0 = the one-block-per-tile k_it_deo2 /
 // k_it_upd_r run.
-static int g_f32p_blocks[64];
+static int g_f32p_blocks[64], g_updr_blocks[64];
 static bool g_f32p_done[64];
 
 template <class K>
@@ -452,8 +452,24 @@ int persist_blocks()
         b = std::min(b, kernel_resident_blocks(k_it_deo2_f32p<kMaxJobs, LF_F32_12>, nsm));
         b = std::min(b, kernel_resident_blocks(k_it_deo2_f32p<kMaxJobs, LF_F16_12>, nsm));
         g_f32p_blocks[dev] = b;
+        int r = kUpdRMinBlocks * nsm;
+        r = std::min(r, kernel_resident_blocks(k_it_upd_r_p<1, VP_DF>, nsm));
+        r = std::min(r, kernel_resident_blocks(k_it_upd_r_p<1, VP_F32>, nsm));
+        r = std::min(r, kernel_resident_blocks(k_it_upd_r_p<kMaxJobs, VP_DF>, nsm));
+        r = std::min(r, kernel_resident_blocks(k_it_upd_r_p<kMaxJobs, VP_F32>, nsm));
+        g_updr_blocks[dev] = r;
+        if (r <= 0) g_f32p_blocks[dev] = 0;
     }
     return g_f32p_blocks[dev];
+}
+
+static int upd_r_blocks()
+{
+    if (persist_blocks() <= 0) return 0;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(g_st_mu);
+    return g_updr_blocks[dev];
 }
 
 // All jobs of the batch carry the staged link stream.
@@ -502,7 +518,7 @@ static void launch_kernel_k(const IterBatch<NJ> &B, int k, int ntot, int vp, int
         if (k == 0 && sb == 0) launch_dep(k_it_deo1<NJ, VP_DF, LF_DF18>, g1, tb, 0, s, dep, B);
         if (k == 1 && sb == 0) launch_dep(k_it_deo2<NJ, VP_DF, LF_DF18>, g1, tb, 0, s, dep, B);
         if (k == 2) {
-            const int pb = std::min(ntot, persist_blocks());
+            const int pb = std::min(ntot, upd_r_blocks());
             if (pb > 0) launch_dep(k_it_upd_r_p<NJ, VP_DF>, dim3((unsigned)pb), tb, 0, s, dep, B, ntot);
             else launch_dep(k_it_upd_r<NJ, VP_DF>, g1, tb, 0, s, dep, B);
         }
@@ -530,7 +546,7 @@ static void launch_kernel_k(const IterBatch<NJ> &B, int k, int ntot, int vp, int
         }
     }
     if (k == 2) {
-        const int pb = std::min(ntot, persist_blocks());
+        const int pb = std::min(ntot, upd_r_blocks());
         if (pb > 0) launch_dep(k_it_upd_r_p<NJ, VP_F32>, dim3((unsigned)pb), tb, 0, s, dep, B, ntot);
         else launch_dep(k_it_upd_r<NJ, VP_F32>, g1, tb, 0, s, dep, B);
     }
@@ -689,8 +705,16 @@ static int link_fmt_for(const lqcd_ctx *c, int prec, const void **links)
     return LF_F32_18;
 }
 
+// FP32 / FP16 links of up to this many bytes keep their place in L2 (129 MB)
+// from one stencil to the next: 24^4 with 12-real FP32 links (64 MB), mixed
+// 15-shift solve 255 -> 240 ms.  Larger sets only evict the vectors: 24^4 with
+// 18 reals (96 MB) K1 27.2 -> 30.4 us, 32^4 with 12 (201 MB) 46.2 -> 50.8.
+constexpr size_t kKeepLinkBytes = (size_t)72 << 20;
+
 static void fill_job(lqcd_ctx *c, const WsPtrs &P, const void *links, IterJob &J)
 {
+    const size_t link = links == c->lnk_h12.ptr ? 24 : (links == c->lnk_f12.ptr ? 48 : (links == c->lnk_f18.ptr ? 72 : 144));
+    J.keep = 8 * c->Vh * link <= kKeepLinkBytes;
     J.g = c->g;
     J.links = links;
     // the staged stream holds the df64 links: only the FP64 engine uses it

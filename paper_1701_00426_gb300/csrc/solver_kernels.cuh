@@ -415,7 +415,15 @@ __device__ __forceinline__ double block_reduce_acc_n(Acc2 A, double *smem)
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// L2 priority of a job's FP32 / FP16 links.
+__device__ __forceinline__ uint64_t link_policy(const IterJob &J)
+{
+    return J.keep ? l2_normal_policy() : l2_evict_first_policy();
+}
+
 // ------------------------------------------------------------------ K1
+// FP16 links: direction loop unrolled, so that later hops' loads go out early
+// (32^4 36.7 -> 34.5 us, 48^4 138 -> 126); with FP32 links it gains nothing.
 template <int NJ, int VP, int LF>
 __global__ void __launch_bounds__(kIterThreads, LQCD_ITER_MINB) k_it_deo1(const __grid_constant__ IterBatch<NJ> B)
 {
@@ -444,7 +452,7 @@ __global__ void __launch_bounds__(kIterThreads, LQCD_ITER_MINB) k_it_deo1(const 
             t[(size_t)c * Vh + i] = make_float4(res[2 * c].x, res[2 * c].y, res[2 * c + 1].x, res[2 * c + 1].y);
     } else {
         float2 o[3];
-        deo_site_f32<LF>(J.g, J.links, p, S, i, 1, Vh, o);
+        deo_site_f32<LF, LF == LF_F16_12 ? 4 : 1>(J.g, J.links, p, S, i, 1, Vh, o, link_policy(J));
 #pragma unroll
         for (int c = 0; c < 3; ++c) t[(size_t)c * Vh + i] = o[c];
     }
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(kIterThreads, LQCD_ITER_MINB) k_it_deo2(const 
             }
         } else {
             float2 o[3];
-            deo_site_f32<LF>(J.g, J.links, (const float2 *)J.t, S, i, 0, Vh, o);
+            deo_site_f32<LF>(J.g, J.links, (const float2 *)J.t, S, i, 0, Vh, o, link_policy(J));
             const float a = st->a0_df.x;
             float d = 0.f;
 #pragma unroll

@@ -27,7 +27,12 @@
 
 namespace lqcd {
 
-constexpr int kF32PersistMinBlocks = 4;  // resident blocks per SM asked of the compiler
+// Resident blocks per SM asked of the compiler.  K2 with three blocks has the
+// registers to issue two directions' loads together; against four blocks and a
+// rolled direction loop: 27.2 -> 24.4 us at 24^4, 49.3 -> 46.9 at 32^4, 201 ->
+// 193 at 48^4 (FP32 12-real).  K3 streams: four (48^4: 43.1 us with three, 40.7).
+constexpr int kF32PersistMinBlocks = 3;
+constexpr int kUpdRMinBlocks = 4;
 
 // Tail of a persistent reduction kernel. Thread 0 takes one ticket per job
 // the block worked on (sh.cnt), after one fence. For every job whose tile
@@ -107,7 +112,7 @@ __global__ void __launch_bounds__(kIterThreads, kF32PersistMinBlocks)
 #pragma unroll
             for (int c = 0; c < 3; ++c) pp[c] = p[(size_t)c * Vh + i];
             float2 o[3];
-            deo_site_f32<LF>(J.g, J.links, (const float2 *)J.t, S, i, 0, Vh, o);
+            deo_site_f32<LF, 2>(J.g, J.links, (const float2 *)J.t, S, i, 0, Vh, o, link_policy(J));
             float2 *q = (float2 *)J.q;
             const float a = st->a0_df.x;
             float d = 0.f;
@@ -144,7 +149,7 @@ __global__ void __launch_bounds__(kIterThreads, kF32PersistMinBlocks)
 // (finalize_rr_warp) in the block that completes the job.  The per-site
 // arithmetic is that of k_it_upd_r.
 template <int NJ, int VP>
-__global__ void __launch_bounds__(kIterThreads, kF32PersistMinBlocks)
+__global__ void __launch_bounds__(kIterThreads, kUpdRMinBlocks)
     k_it_upd_r_p(const __grid_constant__ IterBatch<NJ> B, int ntot)
 {
     using T = typename VecT<VP>::T;
