@@ -8,7 +8,10 @@
 #include <cstring>
 #include <atomic>
 #include <string>
+#include <thread>
 #include <vector>
+
+#include <unistd.h>
 
 #include "internal.h"
 
@@ -44,6 +47,33 @@ void register_bounds_reader(BoundsReader f) { bounds_readers().push_back(f); }
 // Host-side fault injection (lqcd_inject_alloc_failure): the k-th device
 // allocation from now fails as cudaMalloc would.
 static std::atomic<long> g_fail_alloc{0};
+
+void prefault_host(void *p, size_t bytes)
+{
+    constexpr size_t kMin = (size_t)4 << 20;
+    if (bytes < kMin) return;
+    const long ps = sysconf(_SC_PAGESIZE);
+    const size_t page = ps > 0 ? (size_t)ps : 4096;
+    auto touch = [=](size_t lo, size_t hi) {
+        for (size_t o = lo; o < hi; o += page) ((volatile char *)p)[o] = 0;
+    };
+    const unsigned hw = std::thread::hardware_concurrency();
+    const size_t nt = std::min({(size_t)8, (size_t)std::max(1u, hw / 2), bytes / kMin});
+    const size_t share = ((bytes / nt) / page + 1) * page;
+    std::vector<std::thread> th;
+    size_t done = 0;   // bytes handed to threads
+    try {
+        th.reserve(nt);
+        for (size_t k = 0; k + 1 < nt && done + share < bytes; ++k) {
+            th.emplace_back(touch, done, done + share);
+            done += share;
+        }
+    } catch (...) {
+        // no more threads or memory: the caller's thread takes the rest
+    }
+    touch(done, bytes);
+    for (std::thread &t : th) t.join();
+}
 
 int DevBuf::ensure(size_t n)
 {

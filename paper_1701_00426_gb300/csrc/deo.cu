@@ -246,6 +246,7 @@ int download_links(lqcd_ctx *c, double *host, size_t n)
     k_links_to_canonical<<<(unsigned)((4 * V + 255) / 256), 256, 0, c->stream>>>(c->g, c->lnk_nat.as<double2>(),
                                                                               stage.as<double2>(), V);
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) prefault_host(host, want * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, stage.ptr, want * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     stage.release();
@@ -291,6 +292,7 @@ int soa_to_host(lqcd_ctx *c, const double2 *dev_soa, double *host, int nf, cudaS
     const long n = (long)c->Vh * nf;
     k_soa_to_aos<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dev_soa, c->io_b.as<double2>(), (long)c->Vh, nf);
     LQCD_CUDA(cudaGetLastError());
+    prefault_host(host, bytes);
     LQCD_CUDA(cudaMemcpyAsync(host, c->io_b.ptr, bytes, cudaMemcpyDeviceToHost, s));
     return LQCD_OK;
 }

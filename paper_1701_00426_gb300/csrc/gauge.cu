@@ -1971,6 +1971,7 @@ int lqcd_mom_download(lqcd_ctx *c, double *H, size_t n)
     else
         k_mom_to_canonical<double><<<nb, 256, 0, c->stream>>>(link_geo(c), c->mom64.as<double>(), stage.as<double2>(), (long)c->V);
     cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) prefault_host(H, want * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpyAsync(H, stage.ptr, want * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     stage.release();
@@ -2156,6 +2157,7 @@ int lqcd_stout_force(lqcd_ctx *c, const double *F_smeared, double *F_thin, size_
                                                                             (long)c->V);
     c->launches += 1;
     e = cudaGetLastError();
+    if (e == cudaSuccess) prefault_host(F_thin, want * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpyAsync(F_thin, stage.ptr, want * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "force download");

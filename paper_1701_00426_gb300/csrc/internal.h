@@ -76,6 +76,12 @@ int cuda_fail(cudaError_t e, const char *what);
         if (_e != cudaSuccess) return ::lqcd::cuda_fail(_e, #call);         \
     } while (0)
 
+// Makes the pages of a host output buffer resident, on several threads: a copy
+// into a fresh array otherwise takes its page faults one by one (127 MB: 20
+// against 187 GB/s into resident pages).  Every byte of the buffer must be
+// about to be written; buffers below 4 MB are left alone.
+void prefault_host(void *p, size_t bytes);
+
 // ------------------------------------------------------------------ device buffer
 struct DevBuf {
     void *ptr = nullptr;
