@@ -29,6 +29,7 @@ struct SolverState {
     int shift_iters[kMaxShifts];
     double last_sum;                  // last reduction result (diagnostics)
     int stall;                        // a staged stencil wait ran out (turned into HALT_STALL)
+    double ratio[kMaxShifts];         // zeta_new / zeta of the active shifts (split finalisers)
     // split copies for the vector kernels: df64 (hi, lo) and FP32 (hi only)
     float2 a0_df, alpha_df;
     float2 alpha_s_df[kMaxShifts], zeta_new_df[kMaxShifts], beta_s_df[kMaxShifts];
@@ -50,6 +51,7 @@ struct IterJob {
     double *part;        // per-tile partial sums
     unsigned *ticket;    // last-block-done counter
     int tile0, ntiles;
+    int split;           // K2's finaliser forms alpha only; a block of K3 forms the shifted coefficients
     int keep;            // FP32 / FP16 links stay in L2 between the stencils: normal priority instead of evict-first
 };
 

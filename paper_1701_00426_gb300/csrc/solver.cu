@@ -519,7 +519,7 @@ static void launch_kernel_k(const IterBatch<NJ> &B, int k, int ntot, int vp, int
         if (k == 1 && sb == 0) launch_dep(k_it_deo2<NJ, VP_DF, LF_DF18>, g1, tb, 0, s, dep, B);
         if (k == 2) {
             const int pb = std::min(ntot, upd_r_blocks());
-            if (pb > 0) launch_dep(k_it_upd_r_p<NJ, VP_DF>, dim3((unsigned)pb), tb, 0, s, dep, B, ntot);
+            if (pb > 0) launch_dep(k_it_upd_r_p<NJ, VP_DF>, dim3((unsigned)(pb + B.njobs)), tb, 0, s, dep, B, ntot);
             else launch_dep(k_it_upd_r<NJ, VP_DF>, g1, tb, 0, s, dep, B);
         }
         if (k == 3) launch_dep(k_it_upd_shifts<NJ, VP_DF>, g1, tb, 0, s, dep, B);
@@ -547,7 +547,7 @@ static void launch_kernel_k(const IterBatch<NJ> &B, int k, int ntot, int vp, int
     }
     if (k == 2) {
         const int pb = std::min(ntot, upd_r_blocks());
-        if (pb > 0) launch_dep(k_it_upd_r_p<NJ, VP_F32>, dim3((unsigned)pb), tb, 0, s, dep, B, ntot);
+        if (pb > 0) launch_dep(k_it_upd_r_p<NJ, VP_F32>, dim3((unsigned)(pb + B.njobs)), tb, 0, s, dep, B, ntot);
         else launch_dep(k_it_upd_r<NJ, VP_F32>, g1, tb, 0, s, dep, B);
     }
     if (k == 3) launch_dep(k_it_upd_shifts<NJ, VP_F32>, g1, tb, 0, s, dep, B);
@@ -714,6 +714,7 @@ constexpr size_t kKeepLinkBytes = (size_t)72 << 20;
 static void fill_job(lqcd_ctx *c, const WsPtrs &P, const void *links, IterJob &J)
 {
     const size_t link = links == c->lnk_h12.ptr ? 24 : (links == c->lnk_f12.ptr ? 48 : (links == c->lnk_f18.ptr ? 72 : 144));
+    J.split = upd_r_blocks() > 0;   // the persistent K3 runs
     J.keep = 8 * c->Vh * link <= kKeepLinkBytes;
     J.g = c->g;
     J.links = links;

@@ -249,6 +249,35 @@ __device__ inline void finalize_pq_warp(SolverState *st, double pq)
     finalize_pq_shifts(st, c);
 }
 
+// The finaliser of K2's last block: alpha and, unless a block of K3 does it,
+// the shifted coefficients.
+__device__ __forceinline__ void finalize_pq_job(const IterJob &J, double pq)
+{
+    const PqCarry c = finalize_pq_alpha(J.st, pq);
+    if (!J.split) finalize_pq_shifts(J.st, c);
+}
+
+// The shifted coefficients in the kernel after the one that formed alpha (one
+// warp): what finalize_pq_alpha loaded is still in the state, the old alpha and
+// beta as alpha_prev and beta_prev.  Also zeta_new / zeta, which the
+// coefficients beta_i need.
+__device__ __forceinline__ void finalize_pq_late(SolverState *st)
+{
+    const int lane = threadIdx.x & 31;
+    PqCarry c;
+    c.alpha = st->alpha;
+    c.alpha_old = st->alpha_prev;
+    c.beta_old = st->beta_prev;
+    c.act = (lane < st->n_shift) ? st->active_next[lane] : 0;
+    c.zo = st->zeta[lane];
+    c.zc = st->zeta_new[lane];
+    c.srel = st->shift_rel[lane];
+    c.m = __ballot_sync(0xFFFFFFFFu, c.act);
+    c.ok = true;
+    finalize_pq_shifts(st, c);
+    if (c.act) st->ratio[lane] = st->zeta_new[lane] / c.zc;
+}
+
 // finalize_rr on one warp: lane k handles the k-th active shift (beta_i and
 // the convergence test); lane 0 the base scalars and the halt decision.
 // Called by warp 0 of the last block.  In two parts: what does not depend on
@@ -258,6 +287,7 @@ struct RrCarry {
     int s, its, iters, n_act, base, max_iter;
 };
 
+template <bool SPLIT = false>
 __device__ __forceinline__ RrCarry finalize_rr_begin(const SolverState *st)
 {
     const int lane = threadIdx.x & 31;
@@ -275,10 +305,11 @@ __device__ __forceinline__ RrCarry finalize_rr_begin(const SolverState *st)
     c.s = st->act_list[lane] & (kMaxShifts - 1);
     const double zc_l = st->zeta[lane], zn_l = st->zeta_new[lane];
     const int it_l = st->shift_iters[lane];
+    const double rt_l = SPLIT ? st->ratio[lane] : 0.0;
     const double zc = __shfl_sync(0xFFFFFFFFu, zc_l, c.s);
     c.zn = __shfl_sync(0xFFFFFFFFu, zn_l, c.s);
     c.its = __shfl_sync(0xFFFFFFFFu, it_l, c.s);
-    c.ratio = c.zn / zc;
+    c.ratio = SPLIT ? __shfl_sync(0xFFFFFFFFu, rt_l, c.s) : c.zn / zc;
     return c;
 }
 
@@ -516,7 +547,7 @@ __global__ void __launch_bounds__(kIterThreads, LQCD_ITER_MINB) k_it_deo2(const 
     }
     const double v = block_reduce_acc_n<kIterThreads>(dot, s_red);
     tile_finish_block(J, tile, v, [&](double tot) {
-        if (threadIdx.x < 32) finalize_pq_warp(st, tot);
+        if (threadIdx.x < 32) finalize_pq_job(J, tot);
     });
 }
 
@@ -713,7 +744,7 @@ __device__ __forceinline__ void k2_staged_consume(RingDF &R, K2Shared &sh, const
             *J.ticket = 0u;
         }
         consumer_sync();
-        if (threadIdx.x < 32) finalize_pq_warp(J.st, sh.tot);
+        if (threadIdx.x < 32) finalize_pq_job(J, sh.tot);
         __threadfence();
         consumer_sync();
     }

@@ -38,8 +38,9 @@ constexpr int kUpdRMinBlocks = 4;
 // the block worked on (sh.cnt), after one fence. For every job whose tile
 // count this block completes, the block sums the tile partials in tile
 // order (the order of tile_finish_block) and warp 0 runs fin(state, total).
+// extra: tickets of a job beyond its tiles.
 template <int NJ, class Fin>
-__device__ __forceinline__ void persist_finish(K2Shared &sh, const IterBatch<NJ> &B, Fin fin)
+__device__ __forceinline__ void persist_finish(K2Shared &sh, const IterBatch<NJ> &B, unsigned extra, Fin fin)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
@@ -49,7 +50,7 @@ __device__ __forceinline__ void persist_finish(K2Shared &sh, const IterBatch<NJ>
             const unsigned n = sh.cnt[j];
             if (!n) continue;
             const unsigned prev = atomicAdd(B.job[j].ticket, n);
-            if (prev + n == (unsigned)B.job[j].ntiles) last |= 1ull << j;
+            if (prev + n == (unsigned)B.job[j].ntiles + extra) last |= 1ull << j;
         }
         sh.last = last;
     }
@@ -73,7 +74,7 @@ __device__ __forceinline__ void persist_finish(K2Shared &sh, const IterBatch<NJ>
             *J.ticket = 0u;
         }
         __syncthreads();
-        if (threadIdx.x < 32) fin(J.st, sh.tot);
+        if (threadIdx.x < 32) fin(J, sh.tot);
         __threadfence();
         __syncthreads();
     }
@@ -142,12 +143,16 @@ __global__ void __launch_bounds__(kIterThreads, kF32PersistMinBlocks)
         }
         ++nb;
     }
-    persist_finish(sh, B, [](SolverState *st, double tot) { finalize_pq_warp(st, tot); });
+    persist_finish(sh, B, 0u, [](const IterJob &J, double tot) { finalize_pq_job(J, tot); });
 }
 
 // K3: r -= alpha q, ||r||^2 per tile, then beta and the convergence tests
 // (finalize_rr_warp) in the block that completes the job.  The per-site
-// arithmetic is that of k_it_upd_r.
+// arithmetic is that of k_it_upd_r.  The last B.njobs blocks of the grid take
+// no tiles: each forms one job's shifted coefficients (two FP64 divisions and
+// their scalars, about 2.5 us on this chip) while the others stream r, instead
+// of K2's finaliser doing it with the whole device waiting, and counts as one
+// more ticket of the job.
 template <int NJ, int VP>
 __global__ void __launch_bounds__(kIterThreads, kUpdRMinBlocks)
     k_it_upd_r_p(const __grid_constant__ IterBatch<NJ> B, int ntot)
@@ -159,10 +164,20 @@ __global__ void __launch_bounds__(kIterThreads, kUpdRMinBlocks)
     dep_launch();
     if (threadIdx.x < NJ) sh.cnt[threadIdx.x] = 0u;
     __syncthreads();
+    const int nblk = (int)gridDim.x - B.njobs;
+    if ((int)blockIdx.x >= nblk) {
+        const int j = (int)blockIdx.x - nblk;
+        if (!B.job[j].st->halt) {
+            if (threadIdx.x < 32) finalize_pq_late(B.job[j].st);
+            __syncthreads();   // warp 0's writes before thread 0's fence and ticket
+            if (threadIdx.x == 0) sh.cnt[j] = 1u;
+        }
+        __syncthreads();
+    }
     // The block's tiles of live jobs; each tile's r and q are loaded while
     // the previous tile's norm is reduced.
     auto next_live = [&](int gt) -> int {
-        for (; gt < ntot; gt += gridDim.x) {
+        for (; gt < ntot; gt += nblk) {
             int j, tile;
             tile_of(B, gt, j, tile);
             if (!B.job[j].st->halt) return gt;
@@ -185,7 +200,7 @@ __global__ void __launch_bounds__(kIterThreads, kUpdRMinBlocks)
         }
     };
     int nb = 0;
-    int gt = next_live((int)blockIdx.x);
+    int gt = (int)blockIdx.x < nblk ? next_live((int)blockIdx.x) : -1;
     if (gt >= 0) load_rq(gt);
     while (gt >= 0) {
         int j, tile;
@@ -222,7 +237,7 @@ __global__ void __launch_bounds__(kIterThreads, kUpdRMinBlocks)
                 nrm.s = d;
             }
         }
-        const int gn = next_live(gt + (int)gridDim.x);
+        const int gn = next_live(gt + nblk);
         if (gn >= 0) load_rq(gn);
         const int b = nb & 1;  // double-buffered warp sums, as in k_it_deo2_f32p
         warp_reduce_acc(nrm);
@@ -238,7 +253,10 @@ __global__ void __launch_bounds__(kIterThreads, kUpdRMinBlocks)
         ++nb;
         gt = gn;
     }
-    persist_finish(sh, B, [](SolverState *st, double tot) { finalize_rr_warp(st, tot); });
+    persist_finish(sh, B, 1u, [](const IterJob &J, double tot) {
+        const RrCarry c = finalize_rr_begin<true>(J.st);
+        finalize_rr_end(J.st, c, tot);
+    });
 }
 
 }  // namespace lqcd
