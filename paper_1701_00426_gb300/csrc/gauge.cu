@@ -130,17 +130,52 @@ __device__ __forceinline__ SiteIdx site_step(const LinkGeo &g, const int (&x)[4]
     return s;
 }
 
-// U_dir at a site, or its conjugate transpose (read transposed, imaginary parts
-// negated).
-template <class T>
-__device__ __forceinline__ void link_or_dag(const typename Vec2T<T>::t *__restrict__ L, int dir, SiteIdx s, int Vh,
-                                            bool dag, Mat3<T> &U)
+// Lexicographic offset of d steps in direction m from x.  Offsets of different
+// directions add, so a site of a staple costs one addition.
+__device__ __forceinline__ int step_delta(const LinkGeo &g, const int (&x)[4], int m, int d)
 {
-    const typename Vec2T<T>::t *p = L + (size_t)((dir * 2 + s.par) * 9) * Vh + s.idx;
-    const size_t row = (size_t)(dag ? 1 : 3) * Vh, col = (size_t)(dag ? 3 : 1) * Vh;
+    const int n = g.N[m], v = m == 0 ? x[0] : m == 1 ? x[1] : m == 2 ? x[2] : x[3];
+    const int stride = m == 0 ? 1 : g.N[0] * (m == 1 ? 1 : g.N[1] * (m == 2 ? 1 : g.N[2]));
+    return (wrap(v + d, n) - v) * stride;
+}
+
+// Links on their way from L2 to a thread: D slots of nine components per thread
+// of the block, filled with cp.async.  A thread reads only what it copied.
+template <class T>
+struct LinkRing {
+    static constexpr int D = sizeof(T) == 4 ? 4 : 2;
+    static constexpr bool keep = sizeof(T) == 4;   // one more slot, for the link that every side takes
+    typename Vec2T<T>::t e[D + (keep ? 1 : 0)][9][kGaugeThreads];
+};
+
+// U_dir at a site into slot (one group; an empty one if !live)
+template <class T>
+__device__ __forceinline__ void ring_fetch(LinkRing<T> &R, int slot, const typename Vec2T<T>::t *__restrict__ L, int dir,
+                                           SiteIdx s, int Vh, bool live = true)
+{
+    using V = typename Vec2T<T>::t;
+    if (live) {
+        const unsigned off = ((unsigned)((dir * 2 + s.par) * 9) * (unsigned)Vh + (unsigned)s.idx);
+        const unsigned d = (unsigned)__cvta_generic_to_shared(&R.e[slot][0][threadIdx.x]);
+#pragma unroll
+        for (int c = 0; c < 9; ++c)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d + c * (unsigned)(kGaugeThreads * sizeof(V))),
+                         "l"(L + (size_t)c * Vh + off), "n"
+                         (sizeof(V))
+                         : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The link in a slot, or its conjugate transpose (read transposed, imaginary
+// parts negated).
+template <class T>
+__device__ __forceinline__ void ring_read(const LinkRing<T> &R, int slot, bool dag, Mat3<T> &U)
+{
+    const int row = dag ? 1 : 3, col = dag ? 3 : 1;
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
-        const typename Vec2T<T>::t v = __ldg(p + (c / 3) * row + (c % 3) * col);
+        const typename Vec2T<T>::t v = R.e[slot][(c / 3) * row + (c % 3) * col][threadIdx.x];
         U.e[c] = {v.x, dag ? -v.y : v.y};
     }
 }
@@ -163,61 +198,107 @@ __device__ __forceinline__ void coords_of(const LinkGeo &g, int P, int i, int (&
 // Q U_mu(x-mu+s nu)^dag (step -s nu) U_mu(x-mu), rectangles (a) and (c)
 // end in E, so c0 Q + c1 (a' + c') is multiplied by E once.
 // A step in direction -nu starting at y is U_nu(y - nu)^dag.
+// Twelve links of a side come through the ring in the order of their use, D - 1
+// links ahead, across sides.
+constexpr int kSideLinks = 12;
 template <class T>
-__device__ void staple_sum_dev(const LinkGeo &g, const typename Vec2T<T>::t *L, const int (&x)[4], int P, int i, int mu,
-                               Mat3<T> &A)
+__device__ __forceinline__ void staple_sum_dev(const LinkGeo &g, const typename Vec2T<T>::t *__restrict__ L,
+                                               LinkRing<T> &R, const int (&x)[4], int P, int i, int mu, Mat3<T> &A)
 {
+    constexpr int D = LinkRing<T>::D;
     const int Vh = g.Vh;
 #pragma unroll
     for (int k = 0; k < 9; ++k) A.e[k] = {T(0), T(0)};
     const T c0 = T(kSymC0), c1 = T(kSymC1);
-    const SiteIdx s0 = {P, i}, f1 = site_step(g, x, mu, 1), f2 = site_step(g, x, mu, 2), b1 = site_step(g, x, mu, -1);
+    const int full = x[0] + g.N[0] * (x[1] + g.N[1] * (x[2] + g.N[2] * x[3]));
+    const int dm1 = step_delta(g, x, mu, 1), dm2 = step_delta(g, x, mu, 2), db1 = step_delta(g, x, mu, -1);
+    // the site at lexicographic offset d, an odd or even number of steps away
+    auto at = [&](int d, int odd) { return SiteIdx{P ^ odd, bound_index((full + d) >> 1, Vh)}; };
+    // link k of the side (nu, up); d1, d2: offsets of one and two steps s nu
+    auto fetch = [&](int slot, int k, int nu, bool up, int d1, int d2, bool live) {
+        SiteIdx s;
+        int dir = mu;
+        switch (k) {
+            case 0: dir = nu; s = up ? at(dm1, 1) : at(dm1 + d1, 0); break;
+            case 1: s = at(d1, 1); break;
+            case 2: s = at(db1 + d1, 0); break;
+            case 3: dir = nu; s = up ? at(db1, 1) : at(db1 + d1, 0); break;
+            case 4: dir = nu; s = up ? at(dm1 + d1, 0) : at(dm1 + d2, 1); break;
+            case 5: s = at(d2, 0); break;
+            case 6: dir = nu; s = up ? at(d1, 1) : at(d2, 0); break;
+            case 7: s = at(dm1, 1); break;
+            case 8: dir = nu; s = up ? at(dm2, 0) : at(dm2 + d1, 1); break;
+            case 9: s = at(dm1 + d1, 0); break;
+            case 10: s = at(d1, 1); break;
+            default: dir = nu; s = up ? SiteIdx{P, i} : at(d1, 1); break;
+        }
+        ring_fetch<T>(R, slot, L, dir, s, Vh, live);
+    };
+    int w = mu == 0 ? 2 : 0;
+    int d1 = step_delta(g, x, w >> 1, -1);
+    const SiteIdx b1 = at(db1, 1);
+    if (LinkRing<T>::keep) ring_fetch<T>(R, D, L, mu, b1, Vh);   // U_mu(x - mu)
+#pragma unroll
+    for (int k = 0; k < D - 1; ++k) fetch(k, k, w >> 1, false, d1, 0, true);
 #pragma unroll 1
-    for (int w = 0; w < 8; ++w) {
+    while (w < 8) {
         const int nu = w >> 1;
         const bool up = (w & 1) != 0;   // s = -1, then +1
-        if (nu == mu) continue;
-        const int s = up ? 1 : -1;
-        const SiteIdx n1 = site_step(g, x, nu, s), n2 = site_step(g, x, nu, 2 * s);
-        const SiteIdx fn = site_step(g, x, mu, 1, nu, s), bn = site_step(g, x, mu, -1, nu, s);
+        const int d2 = step_delta(g, x, nu, up ? 2 : -2);
+        int wn = w + 1;
+        if ((wn >> 1) == mu) wn += 2;
+        const int nn = min(wn, 7) >> 1;
+        const bool un = (wn & 1) != 0;
+        const int dn = step_delta(g, x, nn, un ? 1 : -1);
+        // link k into U, and the one D - 1 further on into the slot of link k - 1
+        auto take = [&](int k, bool dag, Mat3<T> &U) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(D - 2) : "memory");
+            ring_read<T>(R, k % D, dag, U);
+            const int f = k + D - 1;
+            if (f < kSideLinks) fetch(f % D, f, nu, up, d1, d2, true);
+            else fetch(f % D, f - kSideLinks, nn, un, dn, 0, wn < 8);
+        };
         Mat3<T> P1, Q, W, t1, t2;
         // P1 = step(x+mu, s nu)
-        link_or_dag<T>(L, nu, up ? f1 : fn, Vh, !up, P1);
+        take(0, !up, P1);
         // Q = P1 U_mu(x + s nu)^dag
-        link_or_dag<T>(L, mu, n1, Vh, true, t1);
+        take(1, true, t1);
         mat_mul(P1, t1, Q);
         // rectangle (b): Q U_mu(x - mu + s nu)^dag step(x-mu+s nu, -s nu) U_mu(x - mu)
-        link_or_dag<T>(L, mu, bn, Vh, true, t1);
+        take(2, true, t1);
         mat_mul(Q, t1, t2);
-        link_or_dag<T>(L, nu, up ? b1 : bn, Vh, up, t1);
+        take(3, up, t1);
         mat_mul(t2, t1, W);
-        link_or_dag<T>(L, mu, b1, Vh, false, t1);
+        if (LinkRing<T>::keep) ring_read<T>(R, D, false, t1);
+        else load_link_soa<T>(L, mu, b1.par, b1.idx, Vh, t1);
         mat_mul(W, t1, t2);
         mat_axpy(c1, t2, A);
         // W = c0 Q + c1 (a' + c'), multiplied by E below
 #pragma unroll
         for (int k = 0; k < 9; ++k) W.e[k] = {c0 * Q.e[k].re, c0 * Q.e[k].im};
         // c' = P1 step(x+mu+s nu, s nu) U_mu(x + 2 s nu)^dag step(x + 2 s nu, -s nu)
-        link_or_dag<T>(L, nu, up ? fn : site_step(g, x, mu, 1, nu, -2), Vh, !up, t1);
+        take(4, !up, t1);
         mat_mul(P1, t1, t2);
-        link_or_dag<T>(L, mu, n2, Vh, true, t1);
+        take(5, true, t1);
         mat_mul(t2, t1, Q);
-        link_or_dag<T>(L, nu, up ? n1 : n2, Vh, up, t1);
+        take(6, up, t1);
         mat_mul(Q, t1, t2);
         mat_axpy(c1, t2, W);
         // a' = U_mu(x + mu) step(x + 2 mu, s nu) U_mu(x + mu + s nu)^dag U_mu(x + s nu)^dag
-        link_or_dag<T>(L, mu, f1, Vh, false, P1);
-        link_or_dag<T>(L, nu, up ? f2 : site_step(g, x, mu, 2, nu, -1), Vh, !up, t1);
+        take(7, false, P1);
+        take(8, !up, t1);
         mat_mul(P1, t1, t2);
-        link_or_dag<T>(L, mu, fn, Vh, true, t1);
+        take(9, true, t1);
         mat_mul(t2, t1, Q);
-        link_or_dag<T>(L, mu, n1, Vh, true, t1);
+        take(10, true, t1);
         mat_mul(Q, t1, t2);
         mat_axpy(c1, t2, W);
         // E = step(x + s nu, -s nu);  A += W E
-        link_or_dag<T>(L, nu, up ? s0 : n1, Vh, up, t1);
+        take(11, up, t1);
         mat_mul(W, t1, t2);
         mat_axpy(T(1), t2, A);
+        w = wn;
+        d1 = dn;
     }
 }
 
@@ -955,11 +1036,16 @@ __device__ __forceinline__ const T *mom_ptr(const T *m, int mu, int P, int Vh)
 
 // H_mu(x) -= eps F_mu(x) for every link.  A block holds the four directions of
 // 32 sites (thread = (mu, site), blocks ordered by parity and site): they share
-// most of the links they read, through L1.  Bound by the links' way from L2 and
-// L1 (102 links of 72 bytes per link in FP32).  FP32, against one direction per
-// block and a wrapped coordinate per link read: 862 -> 704 us at 24^4, 2.64 ->
-// 2.18 ms at 32^4.  Three blocks per SM; left to itself the compiler takes 190
-// registers (two blocks: 867 us), and four or five blocks take 767 and 857.
+// most of the links they read, through L1.  Read straight into registers, the
+// links' way from L2 bounds it (some 75 links of 72 bytes per link in FP32, at
+// eleven warps per SM); through the ring their latency is spent under the
+// products, and L1's data path bounds it (81 % busy: in and out of the ring).
+// FP32, one GB300: 32^4 2180 -> 1837 us, 24^4 703 -> 621, 16^4 140 -> 131, a step
+// at 8^4 24.8 -> 22.8.  (One direction per block, no ring: 24^4 862.)  Rings of
+// three and four slots, three and four blocks per SM: 24^4 626 / 621 and 621 /
+// 636; some links through the ring and some straight: 619 to 679, slower at
+// 32^4; bodies of their own for s = -1 and s = +1, without selections, outgrow the
+// instruction cache: 667.
 template <class T>
 __global__ void __launch_bounds__(kGaugeThreads, sizeof(T) == 4 ? 3 : 2)
     k_gauge_mom_update(LinkGeo g, const typename Vec2T<T>::t *__restrict__ L, T *__restrict__ mom, T beta6, T eps)
@@ -972,7 +1058,8 @@ __global__ void __launch_bounds__(kGaugeThreads, sizeof(T) == 4 ? 3 : 2)
     int x[4];
     coords_of(g, P, i, x);
     Mat3<T> A, U, M;
-    staple_sum_dev<T>(g, L, x, P, i, mu, A);
+    __shared__ LinkRing<T> ring;
+    staple_sum_dev<T>(g, L, ring, x, P, i, mu, A);
     load_link_soa<T>(L, mu, P, i, Vh, U);
     mat_mul(U, A, M);
     // F = -(i beta/6)(M - M^dag): F_ij = (beta/6) * (i (conj(M_ji) - M_ij))

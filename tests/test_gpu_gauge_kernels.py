@@ -75,3 +75,23 @@ def test_momentum_update_from_stored_staples(gpu, orc, prec, dims, fail):
             gpu.inject_alloc_failure(0)
         got = c.mom_download()
     assert rel(got - H, ref - H) <= (1e-12 if prec == 0 else 1e-13)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (2, 6, 4, 4), (4, 4, 6, 10), (8, 2, 6, 12)])
+def test_fp32_momentum_update(gpu, orc, dims):
+    """The FP32 force, its links through the per-thread ring, against the FP64
+    oracle: wrapping sides of 2 (a double step returns to the site) and ragged last
+    blocks.  Bar: five products in a row, each 6 roundings of 2^-24 = 6e-8 per
+    entry, 2e-6 at worst; H itself, rounded to FP32 before and after, adds 2 x
+    6e-8 of |H| against |eps F| >= 0.1 |H|, 1.2e-6."""
+    U = inputs.random_links(dims, seed=136)
+    H = inputs.random_momenta(dims, seed=137)
+    eps, beta = 0.5, 5.52
+    ref = orc.mom_update(dims, U, H, beta, eps)
+    assert np.linalg.norm(ref - H) >= 0.1 * np.linalg.norm(H)
+    with gpu.Context(dims) as c:
+        c.links_upload(U)
+        c.mom_upload(H)
+        c.gauge_mom_update(beta, eps, 1)
+        got = c.mom_download()
+    assert rel(got - H, ref - H) <= 3.5e-6
