@@ -220,6 +220,14 @@ __device__ __forceinline__ void acc_prod(Acc2 &A, float ah, float al, float bh, 
     A.c = __fadd_rn(A.c, tmp);
 }
 
+// acc_prod into an accumulator at zero: the sum with it is exact
+__device__ __forceinline__ void acc_first(Acc2 &A, float ah, float al, float bh, float bl)
+{
+    two_prod(ah, bh, A.s, A.c);
+    A.c = __fmaf_rn(ah, bl, A.c);
+    A.c = __fmaf_rn(al, bh, A.c);
+}
+
 // Same, with the small terms collected in a separate per-hop accumulator
 // ch (added into A.c once per hop by acc_flush): fewer roundings at the
 // magnitude of the running error sum.

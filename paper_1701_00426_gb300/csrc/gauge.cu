@@ -331,16 +331,19 @@ __device__ __forceinline__ void dm_mul(const DM3 &a, const DM3 &b, DM3 &c)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             Acc2 re, im;
-            acc_zero(re);
-            acc_zero(im);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const DC x = a.e[i * 3 + k];
                 const DC y = dg ? b.e[j * 3 + k] : b.e[k * 3 + j];
                 const float2 yi = dg ? df_neg(y.im) : y.im;  // conj for the dagger
-                acc_prod(re, x.re.x, x.re.y, y.re.x, y.re.y);
+                if (k == 0) {
+                    acc_first(re, x.re.x, x.re.y, y.re.x, y.re.y);
+                    acc_first(im, x.re.x, x.re.y, yi.x, yi.y);
+                } else {
+                    acc_prod(re, x.re.x, x.re.y, y.re.x, y.re.y);
+                    acc_prod(im, x.re.x, x.re.y, yi.x, yi.y);
+                }
                 acc_prod(re, -x.im.x, -x.im.y, yi.x, yi.y);
-                acc_prod(im, x.re.x, x.re.y, yi.x, yi.y);
                 acc_prod(im, x.im.x, x.im.y, y.re.x, y.re.y);
             }
             c.e[i * 3 + j].re = acc_result(re);
@@ -348,50 +351,55 @@ __device__ __forceinline__ void dm_mul(const DM3 &a, const DM3 &b, DM3 &c)
         }
 }
 
-// a <- a b, row by row (a row of the product needs only that row of a), so that
-// no third matrix is live
-__device__ __forceinline__ void mm_inplace(DM3 &a, const DM3 &b)
+// r = x b for a row x.  The first product of a sum skips the addition to zero
+// (8 of 78 instructions of a component).
+__device__ __forceinline__ void mm_row(const DC (&x)[3], const DM3 &b, DC (&r)[3])
 {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        DC r[3];
+    for (int j = 0; j < 3; ++j) {
+        Acc2 re, im;
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            Acc2 re, im;
-            acc_zero(re);
-            acc_zero(im);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const DC x = a.e[i * 3 + k], y = b.e[k * 3 + j];
-                acc_prod(re, x.re.x, x.re.y, y.re.x, y.re.y);
-                acc_prod(re, -x.im.x, -x.im.y, y.im.x, y.im.y);
-                acc_prod(im, x.re.x, x.re.y, y.im.x, y.im.y);
-                acc_prod(im, x.im.x, x.im.y, y.re.x, y.re.y);
+        for (int k = 0; k < 3; ++k) {
+            const DC y = b.e[k * 3 + j];
+            if (k == 0) {
+                acc_first(re, x[k].re.x, x[k].re.y, y.re.x, y.re.y);
+                acc_first(im, x[k].re.x, x[k].re.y, y.im.x, y.im.y);
+            } else {
+                acc_prod(re, x[k].re.x, x[k].re.y, y.re.x, y.re.y);
+                acc_prod(im, x[k].re.x, x[k].re.y, y.im.x, y.im.y);
             }
-            r[j].re = acc_result(re);
-            r[j].im = acc_result(im);
+            acc_prod(re, -x[k].im.x, -x[k].im.y, y.im.x, y.im.y);
+            acc_prod(im, x[k].im.x, x[k].im.y, y.re.x, y.re.y);
         }
+        r[j].re = acc_result(re);
+        r[j].im = acc_result(im);
+    }
+}
+__device__ __forceinline__ void mm_row(const Cplx<double> (&x)[3], const Mat3<double> &b, Cplx<double> (&r)[3])
+{
 #pragma unroll
-        for (int j = 0; j < 3; ++j) a.e[i * 3 + j] = r[j];
+    for (int j = 0; j < 3; ++j) {
+        double re = 0, im = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const Cplx<double> y = b.e[k * 3 + j];
+            re = fma(x[k].re, y.re, fma(-x[k].im, y.im, re));
+            im = fma(x[k].re, y.im, fma(x[k].im, y.re, im));
+        }
+        r[j] = {re, im};
     }
 }
 
-__device__ __forceinline__ void mm_inplace(Mat3<double> &a, const Mat3<double> &b)
+// a <- a b, row by row (a row of the product needs only that row of a), so that
+// no third matrix is live
+template <class R>
+__device__ __forceinline__ void mm_inplace(Mat3<R> &a, const Mat3<R> &b)
 {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-        Cplx<double> r[3];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            double re = 0, im = 0;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                const Cplx<double> x = a.e[i * 3 + k], y = b.e[k * 3 + j];
-                re = fma(x.re, y.re, fma(-x.im, y.im, re));
-                im = fma(x.re, y.im, fma(x.im, y.re, im));
-            }
-            r[j] = {re, im};
-        }
+        Cplx<R> r[3];
+        const Cplx<R> x[3] = {a.e[i * 3], a.e[i * 3 + 1], a.e[i * 3 + 2]};
+        mm_row(x, b, r);
 #pragma unroll
         for (int j = 0; j < 3; ++j) a.e[i * 3 + j] = r[j];
     }
@@ -831,15 +839,21 @@ __device__ __forceinline__ void load_side(const float4 *__restrict__ L, int k, S
         U.e[c].im = xor_sign(make_float2(v.z, v.w), neg);
     }
 }
+// the sign bit on the integer pipe: a negation is an FP64 instruction
+__device__ __forceinline__ double flip_sign(double a, uint32_t neg)
+{
+    return __hiloint2double(__double2hiint(a) ^ (int)neg, __double2loint(a));
+}
 __device__ __forceinline__ void load_side(const double2 *__restrict__ L, int k, SiteIdx s, int Vh, bool dag,
                                           Mat3<double> &U)
 {
     const double2 *p = L + (size_t)((k * 2 + s.par) * 9) * Vh + s.idx;
+    const uint32_t neg = dag ? 0x80000000u : 0u;
     const size_t row = (size_t)(dag ? 1 : 3) * Vh, col = (size_t)(dag ? 3 : 1) * Vh;
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
         const double2 v = __ldg(p + (c / 3) * row + (c % 3) * col);
-        U.e[c] = {v.x, dag ? -v.y : v.y};
+        U.e[c] = {v.x, flip_sign(v.y, neg)};
     }
 }
 __device__ __forceinline__ void store_side(float4 *L, int k, SiteIdx s, int Vh, const DM3 &U)
@@ -891,6 +905,24 @@ __device__ __forceinline__ Cplx<double> get_sm(const double2 *s, int c)
     return {v.x, v.y};
 }
 
+__device__ __forceinline__ void put_elem(float4 *s, int c, const DC &v)
+{
+    s[c * kGaugeThreads] = make_float4(v.re.x, v.re.y, v.im.x, v.im.y);
+}
+__device__ __forceinline__ void put_elem(double2 *s, int c, const Cplx<double> &v)
+{
+    s[c * kGaugeThreads] = make_double2(v.re, v.im);
+}
+// an element, conjugated if dag
+__device__ __forceinline__ DC side_elem(const float4 &v, bool dag)
+{
+    return {make_float2(v.x, v.y), xor_sign(make_float2(v.z, v.w), dag ? 0x80000000u : 0u)};
+}
+__device__ __forceinline__ Cplx<double> side_elem(const double2 &v, bool dag)
+{
+    return {v.x, flip_sign(v.y, dag ? 0x80000000u : 0u)};
+}
+
 // Stored staples of the planes pr: thread = (ordered pair (p, q), parity, site);
 // C = U_p(x) U_q(x+p) gives up_qp(x) = C U_p(x+q)^dag and
 // down_pq(x+q) = U_q(x)^dag C.  One product in a loop: unrolled, the
@@ -929,14 +961,23 @@ __global__ void __launch_bounds__(kGaugeThreads, 4)
 
 // H_mu(x) -= eps F of the planes pr from the stored staples (F and the update in
 // FP64).  A block holds the four directions of 32 sites, which share most of
-// the links and staples they read through L1.
+// the links and staples they read through L1.  Bound by the arithmetic: 31
+// products per link, about 1260 FP32 instructions each in double-float, 108 FP64
+// ones natively.  A whole double-float product with its sums is 34 KB of code and
+// misses the instruction cache (a quarter of the warps' time); by rows it is a
+// third of that.  Left factors come by rows too and products go to shared memory,
+// so one register matrix is live.  Momentum update, double-float, one GB300: 16^4
+// 784 -> 645 us, 24^4 3.81 -> 3.06 ms, 32^4 15.5 -> 11.8, 8^4 102 -> 91.  Three and
+// five blocks per SM: 689 and 681 at 16^4.  Native FP64, where the signs of the
+// conjugates moved to the integer pipe: 16^4 2543 -> 2207 us.
 template <class R>
 __global__ void __launch_bounds__(kGaugeThreads, 4)
     k_gauge_mom_sides(LinkGeo g, PlaneRange pr, const typename SideT<R>::t *__restrict__ L,
                       const typename SideT<R>::t *__restrict__ F, double *__restrict__ mom, double beta6, double eps)
 {
     static_assert(kGaugeThreads == 128, "four directions of 32 sites");
-    __shared__ typename SideT<R>::t s_a[9 * kGaugeThreads], s_b[9 * kGaugeThreads];
+    using T = typename SideT<R>::t;
+    __shared__ T s_a[9 * kGaugeThreads], s_b[9 * kGaugeThreads];
     const int Vh = g.Vh, nt = (Vh + 31) / 32;
     const int P = (int)blockIdx.x / nt, i = ((int)blockIdx.x - P * nt) * 32 + ((int)threadIdx.x & 31);
     const int mu = (int)threadIdx.x >> 5;
@@ -944,9 +985,39 @@ __global__ void __launch_bounds__(kGaugeThreads, 4)
     int x[4];
     coords_of(g, P, i, x);
     const SiteIdx s0 = {P, i}, sm = site_step(g, x, mu, 1);
-    typename SideT<R>::t *A = s_a + threadIdx.x, *B = s_b + threadIdx.x;   // sum of the sides; X' Y
-    Mat3<R> M, u;
+    T *A = s_a + threadIdx.x, *B = s_b + threadIdx.x;   // sum of the sides; the product so far
+    Mat3<R> u;
     bool any = false;
+    // D <- X u (+ Y): X number k of S at s (conjugate transposed if dag), or B if !S;
+    // Y = D's place or B, added if add.  Rows in a loop, X's next row loaded before
+    // the products of this one.
+    auto product = [&](const T *S, int k, SiteIdx s, bool dag, const T *Y, bool add, T *D) {
+        const T *p = S ? S + (size_t)((k * 2 + s.par) * 9) * Vh + s.idx : nullptr;
+        const size_t row = (size_t)(dag ? 1 : 3) * Vh, col = (size_t)(dag ? 3 : 1) * Vh;
+        T nx[3];
+        auto fetch = [&](int r) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) nx[c] = S ? __ldg(p + r * row + c * col) : B[(r * 3 + c) * kGaugeThreads];
+        };
+        fetch(0);
+#pragma unroll 1
+        for (int r = 0; r < 3; ++r) {
+            Cplx<R> xr[3], o[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) xr[c] = side_elem(nx[c], dag);
+            if (r < 2) fetch(r + 1);
+            mm_row(xr, u, o);
+            if (add) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const Cplx<R> v = get_sm(Y, r * 3 + c);
+                    o[c] = {r_add(v.re, o[c].re), r_add(v.im, o[c].im)};
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) put_elem(D, r * 3 + c, o[c]);
+        }
+    };
 #pragma unroll 1
     for (int w = 0; w < 8; ++w) {
         const int nu = w >> 1, lower = w & 1;
@@ -959,8 +1030,7 @@ __global__ void __launch_bounds__(kGaugeThreads, 4)
         const int kx = side_of(pr, nu, mu), ky = side_of(pr, mu, nu) + lower;
 #pragma unroll 1
         for (int k = 0; k < 5; ++k) {
-            // left factor: X, X Y, X', X, X' Y + X Y'; right: Y, Z' - 20 Z, Y, Y', Z
-            if (k == 0 || k == 2 || k == 3) load_side(k == 2 ? F : L, k == 2 ? kx : nu, sx, Vh, lower != 0, M);
+            // B = X Y; A += B (Z' - 20 Z); B = X' Y; B += X Y'; A += B Z
             const bool zz = k == 1 || k == 4;
             load_side(k == 3 ? F : L, k == 3 ? ky : (zz ? nu : mu), zz ? sz : sy, Vh, zz ? lower == 0 : true, u);
             if (k == 1) {
@@ -970,35 +1040,21 @@ __global__ void __launch_bounds__(kGaugeThreads, 4)
                 for (int q = 0; q < 9; ++q)
                     u.e[q] = {minus20(z.e[q].re, u.e[q].re), minus20(z.e[q].im, u.e[q].im)};
             }
-            mm_inplace(M, u);
-            if (k == 2) put_sm(B, M);
-            if (k == 3 || k == 4 || k == 1) {
-                // k = 3: M += B; k = 1, 4: A += M
-                if (k == 3 || any) {
-                    const typename SideT<R>::t *y = k == 3 ? B : A;
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        const Cplx<R> v = get_sm(y, q);
-                        M.e[q] = {r_add(v.re, M.e[q].re), r_add(v.im, M.e[q].im)};
-                    }
-                }
-                if (k != 3) {
-                    put_sm(A, M);
-                    any = true;
-                }
-            }
+            T *D = zz ? A : B;
+            product(zz ? nullptr : (k == 2 ? F : L), k == 2 ? kx : nu, sx, !zz && lower != 0, D, k == 3 || (zz && any), D);
+            any |= zz;
         }
     }
     if (!any) return;
-    load_side(L, mu, s0, Vh, false, M);
 #pragma unroll
     for (int q = 0; q < 9; ++q) u.e[q] = get_sm(A, q);
-    mm_inplace(M, u);
+    product(L, mu, s0, false, B, false, B);
     double mre[9], mim[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-        mre[q] = r_double(M.e[q].re);
-        mim[q] = r_double(M.e[q].im);
+        const Cplx<R> v = get_sm(B, q);
+        mre[q] = r_double(v.re);
+        mim[q] = r_double(v.im);
     }
     gauge_kick(mre, mim, mom + (size_t)((mu * 2 + P) * 8) * Vh + i, Vh, beta6 * kSymC1, eps);
 }
