@@ -213,6 +213,15 @@ static __device__ __noinline__ void deo_site_native_from_df(const Geom &g, const
 }
 
 // ------------------------------------------------------------------ native FP64 (reference)
+// a with its sign bit flipped by neg (0 or 1 << 31), on the integer pipe: a product with -1 or
+// a negation is an instruction of the FP64 pipe, which bounds the native kernels
+// (deo_site_nat: 6 of 42 per half-hop; D_oe and D_eo at 24^4 215 -> 187 us, 32^4
+// 611 -> 520, one GB300).
+__device__ __forceinline__ double flip_sign(double a, uint32_t neg)
+{
+    return __hiloint2double(__double2hiint(a) ^ (int)neg, __double2loint(a));
+}
+
 __device__ __forceinline__ void deo_site_nat(const Geom &g, const double2 *L, const double2 *in, const Stencil &S,
                                              int i, int P, int Vh, double2 (&res)[3])
 {
@@ -227,13 +236,13 @@ __device__ __forceinline__ void deo_site_nat(const Geom &g, const double2 *L, co
             const int idx = dir == 0 ? f : b;
             const int par = dir == 0 ? P : 1 - P;
             const int lidx = dir == 0 ? i : b;
-            const double sg = ((dir == 0 ? nf : nb) != 0u) ? -1.0 : 1.0;
+            const uint32_t neg = dir == 0 ? nf : nb;
             const double2 *lp = L + link_base(mu, par, 9, Vh) + lidx;
             double2 v[3], U[9];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const double2 t = ldg2d(in + (size_t)c * Vh + idx);
-                v[c] = make_double2(sg * t.x, sg * t.y);
+                v[c] = make_double2(flip_sign(t.x, neg), flip_sign(t.y, neg));
             }
 #pragma unroll
             for (int c = 0; c < 9; ++c) U[c] = ldg2d(lp + (size_t)c * Vh);

@@ -839,11 +839,6 @@ __device__ __forceinline__ void load_side(const float4 *__restrict__ L, int k, S
         U.e[c].im = xor_sign(make_float2(v.z, v.w), neg);
     }
 }
-// the sign bit on the integer pipe: a negation is an FP64 instruction
-__device__ __forceinline__ double flip_sign(double a, uint32_t neg)
-{
-    return __hiloint2double(__double2hiint(a) ^ (int)neg, __double2loint(a));
-}
 __device__ __forceinline__ void load_side(const double2 *__restrict__ L, int k, SiteIdx s, int Vh, bool dag,
                                           Mat3<double> &U)
 {
