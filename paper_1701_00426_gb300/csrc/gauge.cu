@@ -249,7 +249,8 @@ __device__ __forceinline__ void staple_sum_dev(const LinkGeo &g, const typename 
         if ((wn >> 1) == mu) wn += 2;
         const int nn = min(wn, 7) >> 1;
         const bool un = (wn & 1) != 0;
-        const int dn = step_delta(g, x, nn, un ? 1 : -1);
+        // nothing after the last side (nn may be mu there, whose offsets do not add)
+        const int dn = wn < 8 ? step_delta(g, x, nn, un ? 1 : -1) : 0;
         // link k into U, and the one D - 1 further on into the slot of link k - 1
         auto take = [&](int k, bool dag, Mat3<T> &U) {
             asm volatile("cp.async.wait_group %0;" ::"n"(D - 2) : "memory");
