@@ -37,6 +37,12 @@
  *   - Every call returns an lqcd_status; nothing throws across this ABI.  On
  *     failure lqcd_last_error() describes the cause (thread-local string).
  *   - A context is not thread-safe: one thread at a time per context.
+ *     Several contexts may be driven at once, each by a thread of its own.  A
+ *     solve of a small lattice that is alone on its device keeps most of the
+ *     SMs for up to 256 iterations (about 8 ms) at a time; while calls of other
+ *     threads of the process are in flight that leave it too few SMs, its
+ *     iterations run as separate launches that share the device, with the same
+ *     bits.
  *   - A context lives on the device that was current at lqcd_create.  Every
  *     call that takes a context makes that device current for the call and
  *     restores the calling thread's current device before it returns, so a

@@ -11,6 +11,7 @@
 #include <thread>
 #include <vector>
 
+#include <time.h>
 #include <unistd.h>
 
 #include "internal.h"
@@ -47,6 +48,67 @@ void register_bounds_reader(BoundsReader f) { bounds_readers().push_back(f); }
 // Host-side fault injection (lqcd_inject_alloc_failure): the k-th device
 // allocation from now fails as cudaMalloc would.
 static std::atomic<long> g_fail_alloc{0};
+
+// ------------------------------------------------------------------ calls in flight
+struct alignas(64) DeviceLoad {
+    std::atomic<int> sms{0};             // asked for by the calls in flight
+    std::atomic<long> unfit_ms{-1000000};  // last time a resident launch did not fit beside them
+};
+static DeviceLoad g_load[64];
+static thread_local CallScope *t_scopes = nullptr;   // innermost first
+
+static long coarse_ms()
+{
+    timespec t;
+    clock_gettime(CLOCK_MONOTONIC_COARSE, &t);
+    return (long)t.tv_sec * 1000 + t.tv_nsec / 1000000;
+}
+
+CallScope *CallScope::of(int dev)
+{
+    for (CallScope *s = t_scopes; s; s = s->up_)
+        if (s->dev_ == dev) return s;
+    return nullptr;
+}
+
+CallScope::CallScope(int dev) : dev_(-1)
+{
+    if (dev < 0 || dev >= 64 || of(dev)) return;
+    dev_ = dev;
+    up_ = t_scopes;
+    t_scopes = this;
+    g_load[dev].sms.fetch_add(need_, std::memory_order_relaxed);
+}
+
+CallScope::~CallScope()
+{
+    if (dev_ < 0) return;
+    g_load[dev_].sms.fetch_sub(need_, std::memory_order_relaxed);
+    t_scopes = up_;
+}
+
+void CallScope::declare(int dev, int sms)
+{
+    CallScope *s = of(dev);
+    if (!s) return;
+    g_load[dev].sms.fetch_add(sms - s->need_, std::memory_order_relaxed);
+    s->need_ = sms;
+}
+
+bool CallScope::fits(int dev, int sms, int nsm)
+{
+    if (dev < 0 || dev >= 64) return true;
+    const CallScope *s = of(dev);
+    DeviceLoad &d = g_load[dev];
+    const int others = d.sms.load(std::memory_order_relaxed) - (s ? s->need_ : 0);
+    const long now = coarse_ms();
+    if (others > 0 && others + sms > nsm) {
+        d.unfit_ms.store(now, std::memory_order_relaxed);
+        return false;
+    }
+    // threads that solve in turns leave gaps between their calls
+    return now - d.unfit_ms.load(std::memory_order_relaxed) > kLingerMs;
+}
 
 void prefault_host(void *p, size_t bytes)
 {
@@ -375,6 +437,7 @@ int lqcd_mscg_solve(lqcd_ctx *c, double mass, const double *shifts, int n_shift,
     LQCD_ON_DEVICE(c->device);
     if (!b || !x || !shifts) return fail(LQCD_EINVAL, "NULL argument");
     if (n_shift < 1 || n_shift > LQCD_MAX_SHIFTS) return fail(LQCD_EINVAL, "n_shift must be in 1..32");
+    CallScope::declare(c->device, resident_sms(c));
     const size_t n3 = 3 * c->Vh;
     // the device copies of b and x stay with the context (grown, never shrunk)
     // so that repeated host calls allocate nothing
@@ -400,6 +463,7 @@ int lqcd_mscg_solve_dev(lqcd_ctx *c, double mass, const double *shifts, int n_sh
     NvtxRange nvtx_("lqcd_mscg_solve_dev");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
     LQCD_ON_DEVICE(c->device);
+    CallScope::declare(c->device, resident_sms(c));
     return mscg_solve_dev(c, mass, shifts, n_shift, tol, (const double2 *)b, (double2 *)x, info, (cudaStream_t)stream);
 }
 

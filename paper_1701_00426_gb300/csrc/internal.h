@@ -58,9 +58,40 @@ struct DeviceGuard {
     DeviceGuard &operator=(const DeviceGuard &) = delete;
 };
 
+// SMs that the library calls in flight on a device ask for (api.cu).  A call
+// counts as the whole device unless it declares less.  The resident iteration
+// (resident.cu) holds its SMs for milliseconds, so it runs only while the calls
+// of the other threads leave them free; alone on the device, or with calls that
+// fit beside it, nothing changes.  n threads that solve on one GB300, ms per
+// solve of each, four kernels / resident whatever else runs / with this rule:
+// 12^4 n = 2 23.5 / 26.0 / 22.3, n = 4 25.9 / 52.4 / 25.4; 16^4 n = 4 43.8 / 81.8 /
+// 43.3; 8^4 (64 SMs each) n = 2 22.0 / 11.0 / 10.8, n = 8 30.9 / 46.7 / 28.5; a 24^4
+// solve beside 16^4 ones 69.5 / 83.5 / 69.0.  The linger (threads that solve in a
+// loop leave gaps between their calls) costs one solve's change of form, once.
+struct CallScope {
+    static constexpr int kWhole = 1 << 16;
+    explicit CallScope(int dev);   // within another scope of this thread on the same device: part of that one
+    ~CallScope();
+    CallScope(const CallScope &) = delete;
+    CallScope &operator=(const CallScope &) = delete;
+    // what the calling thread's call on dev asks for from now on
+    static void declare(int dev, int sms);
+    // whether the calls of other threads leave `sms` of the device's nsm free, now
+    // and for the last kLingerMs
+    static bool fits(int dev, int sms, int nsm);
+    static constexpr int kLingerMs = 50;
+
+private:
+    int dev_;        // -1: nothing to undo
+    int need_ = kWhole;
+    CallScope *up_ = nullptr;
+    static CallScope *of(int dev);
+};
+
 // Every C entry point that receives a context (or a server) opens one of
 // these right after its NULL check.
 #define LQCD_ON_DEVICE(dev)                                                               \
+    ::lqcd::CallScope lqcd_call_scope_(dev);                                              \
     ::lqcd::DeviceGuard lqcd_device_guard_(dev);                                          \
     if (!lqcd_device_guard_.ok)                                                           \
         return ::lqcd::fail(LQCD_ECUDA, "cannot make the context's device current")
@@ -260,8 +291,10 @@ int mscg_solve_packed(lqcd_ctx *const *ctxs, int n, const double *mass, const do
                       lqcd_solve_info *info);
 
 // resident.cu: iterations of the batch as cooperative launches until every
-// job halts; done = false: the batch does not take this path.
+// job halts; done = false: the batch does not take this path, or left it between
+// two launches because other threads' calls need the device.
 constexpr int kResSteps = 256;   // iterations of one launch, at most
+int resident_sms(const lqcd_ctx *c);   // SMs that a solve on c asks for (CallScope::declare)
 template <int NJ>
 int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_iter, cudaStream_t s, bool &done);
 

@@ -125,6 +125,15 @@ static int res_share(const IterBatch<NJ> &B, int nblk, int *cta_start)
     return (int)lo;
 }
 
+int resident_sms(const lqcd_ctx *c)
+{
+    const bool df_only = c->opts.prec == LQCD_PREC_FP64;
+    const int nsm = resident_blocks(c->device);
+    if (c->opts.pdl || nsm <= 0 || (long)c->Vh > (df_only ? kResMaxSitesDF : kResMaxSitesF32)) return CallScope::kWhole;
+    const long nsub = ((long)c->Vh + kResSub - 1) / kResSub, m = (nsub + nsm - 1) / nsm;
+    return (int)((nsub + m - 1) / m);   // res_share for one job
+}
+
 template <int NJ>
 int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_iter, cudaStream_t s, bool &done)
 {
@@ -132,7 +141,10 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     if (c->opts.pdl || persist_blocks() <= 0 || kSites != kTile) return LQCD_OK;
     long sites = 0;
     for (int j = 0; j < B.njobs; ++j) sites += B.job[j].g.Vh;
-    if (sites > (vp == VP_DF ? kResMaxSitesDF : kResMaxSitesF32)) return LQCD_OK;
+    if (sites > (vp == VP_DF ? kResMaxSitesDF : kResMaxSitesF32)) {
+        CallScope::declare(c->device, CallScope::kWhole);
+        return LQCD_OK;
+    }
     const int nblk = resident_blocks(c->device);
     ResBatch<NJ> R;
     memset(&R, 0, sizeof R);
@@ -141,6 +153,9 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     R.in_smem = res_smem(vp, lf, m, true) <= kResSmemMax;
     const size_t smem = res_smem(vp, lf, m, R.in_smem != 0);
     if (smem > kResSmemMax) return LQCD_OK;
+    const int blocks = R.cta_start[B.njobs];
+    CallScope::declare(c->device, blocks);
+    if (!CallScope::fits(c->device, blocks, nblk)) return LQCD_OK;
     R.njobs = B.njobs;
     // kResWords words of counts for every job, then the published warp sums
     size_t slots = 0;
@@ -172,7 +187,7 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
         c->res_tag += (uint32_t)R.steps;
         cudaError_t e = cudaMemsetAsync(c->res_xch.ptr, 0, (size_t)B.njobs * kResWords * sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
-        res_launch<NJ>(R, vp, lf, R.cta_start[B.njobs], smem, s);
+        res_launch<NJ>(R, vp, lf, blocks, smem, s);
         e = cudaGetLastError();
         c->launches += 1;
         for (int j = 0; j < B.njobs && e == cudaSuccess; ++j)
@@ -190,7 +205,10 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
         cudaEventDestroy(ev[1]);
         return LQCD_OK;
     }
+    bool shared = false;   // others need the device: the four kernels go on from the end of the last launch
     for (int k = 0; k < max_launches && e == cudaSuccess; ++k) {
+        shared = !CallScope::fits(c->device, blocks, nblk);
+        if (shared) break;
         const int nxt = slot ^ 1;
         e = enqueue(nxt);
         if (e != cudaSuccess) break;
@@ -205,7 +223,7 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
     if (e != cudaSuccess) return cuda_fail(e, "resident iteration");
-    done = true;
+    done = !shared;
     return LQCD_OK;
 }
 

@@ -299,6 +299,7 @@ void lqcd_server::run()
             cv.wait(lk, [&] { return stop || !queue.empty() || !active.empty(); });
             if (stop) break;
         }
+        CallScope scope(device);   // this thread makes CUDA calls until the end of the tick
         admit();
         {
             std::lock_guard<std::mutex> lk(mu);
