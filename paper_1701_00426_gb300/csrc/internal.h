@@ -109,8 +109,8 @@ int cuda_fail(cudaError_t e, const char *what);
 
 // Makes the pages of a host output buffer resident, on several threads: a copy
 // into a fresh array otherwise takes its page faults one by one (127 MB: 20
-// against 187 GB/s into resident pages).  Every byte of the buffer must be
-// about to be written; buffers below 4 MB are left alone.
+// against 187 GB/s into resident pages).  The contents stay as they are;
+// buffers below 4 MB, and those resident already, are left alone.
 void prefault_host(void *p, size_t bytes);
 
 // ------------------------------------------------------------------ device buffer
