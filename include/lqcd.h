@@ -527,6 +527,13 @@ void lqcd_serve_destroy(lqcd_server *srv);
  * usable.  Synchronous. */
 int lqcd_selftest_stage_wait(lqcd_ctx *ctx, double limit_s);
 
+/* The same for the resident iteration of small lattices: two blocks, of which
+ * the second waits, limited to limit_s seconds, first at a barrier that the
+ * other one never reaches and then for a sum that nothing publishes.
+ * Returns what a solve with such a stall returns, LQCD_ETIMEOUT, also where the
+ * block that gave up is not the one that writes the job's state back. */
+int lqcd_selftest_resident_wait(lqcd_ctx *ctx, double limit_s);
+
 /* ---------------------------------------------------------------- stout smearing
  * Stout smearing of the fermion links (Sec. 2.1: stout-improved staggered
  * action, Ref. Morningstar:2003gk; Sec. 2.2: a few stout levels).  One level

@@ -331,7 +331,7 @@ int lqcd_create(const int dims[4], const lqcd_opts *opts, lqcd_ctx **out)
     c->opts = o;
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaStreamCreate(&c->stream);
-    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_pinned, 2 * kMaxJobs * sizeof(int), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_pinned, 3 * kMaxJobs * sizeof(int), cudaHostAllocDefault);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&c->h_pinned_d, 64 * sizeof(double), cudaHostAllocDefault);
     if (e != cudaSuccess) {
         st = cuda_fail(e, "lqcd_create");
@@ -437,6 +437,13 @@ int lqcd_selftest_stage_wait(lqcd_ctx *c, double limit_s)
     if (!c) return fail(LQCD_EINVAL, "NULL context");
     LQCD_ON_DEVICE(c->device);
     return stage_wait_selftest(c, limit_s);
+}
+
+int lqcd_selftest_resident_wait(lqcd_ctx *c, double limit_s)
+{
+    if (!c) return fail(LQCD_EINVAL, "NULL context");
+    LQCD_ON_DEVICE(c->device);
+    return resident_wait_selftest(c, limit_s);
 }
 
 int lqcd_deo_apply_mrhs_layout(lqcd_ctx *c, int out_parity, int n_rhs, int recon, int layout, const void *in,

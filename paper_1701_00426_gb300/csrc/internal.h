@@ -209,7 +209,7 @@ struct lqcd_ctx {
     lqcd::GraphCache graph;
     lqcd::DevBuf res_xch;     // flag words and published warp sums of the resident iteration
     uint32_t res_tag = 0;     // last tag handed to a resident launch
-    int *h_pinned = nullptr;  // pinned host words for halt/iteration polling
+    int *h_pinned = nullptr;  // pinned host words: halts of two launches in flight, then stall words [kMaxJobs]
     double *h_pinned_d = nullptr;
     uint64_t launches = 0;    // library kernels launched on behalf of this context
     // t-slab shard of a global lattice (shard.cu); shard_world = 0: not a shard
@@ -233,6 +233,7 @@ int upload_links(lqcd_ctx *c, const double *host, size_t n);
 // Returns true when they can run on the current device.
 bool staged_deo_ready();
 int stage_wait_selftest(lqcd_ctx *c, double limit_s);
+int resident_wait_selftest(lqcd_ctx *c, double limit_s);
 bool staged_solver_ready();
 int persist_blocks();   // grid of the persistent K2 / K3 reduction kernels on this device (0: one block per tile)
 bool staged_active(const lqcd_ctx *c);   // staged option on and the staged link stream built

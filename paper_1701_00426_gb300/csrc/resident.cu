@@ -134,6 +134,47 @@ int resident_sms(const lqcd_ctx *c)
     return (int)((nsub + m - 1) / m);   // res_share for one job
 }
 
+// One stall word per job, in the context's pinned memory (which the kernels
+// write directly); read when the stream has finished.
+static unsigned *clear_stall_words(lqcd_ctx *c)
+{
+    unsigned *w = (unsigned *)c->h_pinned + 2 * kMaxJobs;
+    std::fill(w, w + kMaxJobs, 0u);
+    return w;
+}
+
+static int check_stall_words(const volatile unsigned *w, int njobs)
+{
+    for (int j = 0; j < njobs; ++j)
+        if (w[j]) return fail(LQCD_ETIMEOUT, "a bounded device wait of the resident iteration ran out");
+    return LQCD_OK;
+}
+
+int resident_wait_selftest(lqcd_ctx *c, double limit_s)
+{
+    if (!(limit_s > 0.0 && limit_s <= 10.0)) return fail(LQCD_EINVAL, "limit must be in (0, 10] seconds");
+    DevBuf d;
+    if (int st = d.ensure(512)) return st;   // [0] barrier count, [32] halt word, [64 ..] a sum, all zero
+    unsigned *stall = clear_stall_words(c), *w = d.as<unsigned>();
+    int status[2] = {LQCD_OK, LQCD_OK};
+    cudaError_t e = cudaSuccess;
+    for (int which = 0; which < 2 && e == cudaSuccess; ++which) {
+        stall[0] = 0u;
+        e = cudaMemsetAsync(w, 0, 512, c->stream);
+        if (e != cudaSuccess) break;
+        k_res_wait_selftest<<<2, kResThreads, 0, c->stream>>>(w, (const ulonglong2 *)(w + 64), stall, (int *)(w + 32),
+                                                              which, (uint64_t)(limit_s * 1e9));
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e == cudaSuccess) status[which] = check_stall_words(stall, 1);
+    }
+    d.release();
+    if (e != cudaSuccess) return cuda_fail(e, "resident wait self-test");
+    for (int st : status)
+        if (st != LQCD_ETIMEOUT) return fail(LQCD_ESTATE, "a wait that nothing ends did not run out");
+    return check_stall_words(stall, 1);
+}
+
 template <int NJ>
 int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_iter, cudaStream_t s, bool &done)
 {
@@ -177,6 +218,8 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     }
     R.steps = kResSteps;
     int *hs = c->h_pinned;
+    unsigned *stall = clear_stall_words(c);
+    R.stall = stall;
     cudaEvent_t ev[2];
     LQCD_CUDA(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
     LQCD_CUDA(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
@@ -223,6 +266,7 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     cudaEventDestroy(ev[0]);
     cudaEventDestroy(ev[1]);
     if (e != cudaSuccess) return cuda_fail(e, "resident iteration");
+    if (int st = check_stall_words(stall, B.njobs)) return st;
     done = !shared;
     return LQCD_OK;
 }

@@ -37,8 +37,10 @@
 // The results are bitwise those of the four-kernel iteration.
 //
 // Every wait is bounded by the global timer; a block whose wait runs out
-// stops, marks the job HALT_STALL and leaves.  The launch is cooperative, so
-// all blocks are resident.  A job's blocks wait only on one another.
+// stops, sets the job's stall word (host memory, which no block ever clears: the
+// first block writes back its own copy of the state, and would undo a mark that
+// another one left there) and leaves.  The launch is cooperative, so all blocks
+// are resident.  A job's blocks wait only on one another.
 #pragma once
 
 #include "bulk.cuh"
@@ -60,6 +62,7 @@ struct ResBatch {
     uint32_t tag0;               // tags of this launch: tag0 + it
     int cta_start[NJ + 1];       // blocks of job j
     ulonglong2 *xch[NJ];         // [2][sub-tiles] published warp sums
+    unsigned *stall;             // [NJ] set to 1 by a block whose wait ran out
     unsigned *bar[NJ];           // counts at words 0 (grid barrier), 32 and 64 (sums published); zero at launch
     IterJob job[NJ];
 };
@@ -134,7 +137,7 @@ __device__ __forceinline__ void red_add(unsigned *p, unsigned n)
 
 // Until *p has reached n, or the time limit has passed (false).
 template <bool ACQ>
-__device__ __forceinline__ bool poll_count(const unsigned *p, unsigned n)
+__device__ __forceinline__ bool poll_count(const unsigned *p, unsigned n, uint64_t limit_ns)
 {
     uint64_t t0 = 0;
     for (unsigned k = 1;; ++k) {
@@ -145,7 +148,7 @@ __device__ __forceinline__ bool poll_count(const unsigned *p, unsigned n)
         if ((k & 63u) == 0u) {
             const uint64_t t = globaltimer_ns();
             if (t0 == 0) t0 = t;
-            if (t - t0 > kStageWaitNs) return false;
+            if (t - t0 > limit_ns) return false;
         }
     }
 }
@@ -153,12 +156,13 @@ __device__ __forceinline__ bool poll_count(const unsigned *p, unsigned n)
 // All blocks of the job have written what they wrote before the call, and
 // this block sees it.  count: barriers passed so far times ncta, plus ncta.
 // Called by every thread.
-__device__ __forceinline__ void res_barrier(ResShared &sh, unsigned *bar, unsigned count)
+__device__ __forceinline__ void res_barrier(ResShared &sh, unsigned *bar, unsigned count,
+                                            uint64_t limit_ns = kStageWaitNs)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-        if (!poll_count<true>(bar, count)) sh.dead = 1;
+        if (!poll_count<true>(bar, count, limit_ns)) sh.dead = 1;
     }
     __syncthreads();
 }
@@ -166,7 +170,7 @@ __device__ __forceinline__ void res_barrier(ResShared &sh, unsigned *bar, unsign
 // Partial total of virtual warp vw (lanes = tiles vw * 32 + lane, strided by
 // 256): the warp's shuffle-tree sum, valid in lane 0.
 __device__ __noinline__ double res_warp_total(ResShared &sh, const ulonglong2 *X, int nsub, int ntiles, uint32_t tag,
-                                                 int vw)
+                                              int vw, uint64_t limit_ns = kStageWaitNs)
 {
     const int lane = threadIdx.x & 31;
     double s = 0.0;
@@ -187,7 +191,7 @@ __device__ __noinline__ double res_warp_total(ResShared &sh, const ulonglong2 *X
                 if ((++tries & 63u) == 0u) {
                     const uint64_t t = globaltimer_ns();
                     if (t0 == 0) t0 = t;
-                    if (t - t0 > kStageWaitNs) {
+                    if (t - t0 > limit_ns) {
                         sh.dead = 1;
                         break;
                     }
@@ -211,7 +215,7 @@ __device__ __noinline__ double res_warp_total(ResShared &sh, const ulonglong2 *X
 // The count carries no ordering: the reader of a sum checks its tags.
 __device__ __forceinline__ void res_counted(ResShared &sh, const unsigned *cnt, unsigned count)
 {
-    if (threadIdx.x == 0 && !poll_count<false>(cnt, count)) sh.dead = 1;
+    if (threadIdx.x == 0 && !poll_count<false>(cnt, count, kStageWaitNs)) sh.dead = 1;
     __syncwarp();
 }
 
@@ -856,17 +860,38 @@ __global__ void __launch_bounds__(kResThreads, 1) k_it_resident(const __grid_con
             if (i < Vh) ((T *)J.r)[(size_t)(k % 3) * Vh + i] = rs[k * 32 + lane];
         }
     }
+    if (stalled && threadIdx.x == 0) {
+        B.stall[j] = 1u;
+        st.stall = 1;
+        st.halt = HALT_STALL;
+    }
     if (cta == 0) {
-        if (stalled && threadIdx.x == 0) {
-            st.stall = 1;
-            st.halt = HALT_STALL;
-        }
         __syncthreads();
         for (int k = (int)threadIdx.x; k < (int)(sizeof(SolverState) / 4); k += kResThreads)
             ((uint32_t *)J.st)[k] = ((const uint32_t *)&st)[k];
-    } else if (stalled && threadIdx.x == 0) {
-        J.st->halt = HALT_STALL;
     }
+}
+
+// The waits with a short limit: block 0 ends at once and marks the job
+// converged, as the first block of a job that missed nothing; block 1 waits for a
+// barrier (which = 0) or a sum (1) that never comes.
+static __global__ void __launch_bounds__(kResThreads, 1)
+    k_res_wait_selftest(unsigned *bar, const ulonglong2 *X, unsigned *stall, int *halt, int which, uint64_t limit_ns)
+{
+    __shared__ ResShared sh;
+    if (threadIdx.x == 0) sh.dead = 0;
+    __syncthreads();
+    if (blockIdx.x == 0) {
+        if (threadIdx.x == 0) *halt = HALT_CONVERGED;
+        return;
+    }
+    if (which == 0) {
+        res_barrier(sh, bar, 2u, limit_ns);
+    } else if (threadIdx.x < 32) {
+        res_warp_total(sh, X, 1, 1, 1u, 0, limit_ns);
+    }
+    __syncthreads();
+    if (sh.dead && threadIdx.x == 0) *stall = 1u;
 }
 
 }  // namespace lqcd

@@ -51,7 +51,7 @@ EXPORTED = [
     "lqcd_mom_upload", "lqcd_mom_download", "lqcd_gauge_mom_update", "lqcd_gauge_link_update",
     "lqcd_gauge_md_steps", "lqcd_gauge_action", "lqcd_mom_energy", "lqcd_fermion_force_update",
     "lqcd_stout_smear", "lqcd_stout_restore", "lqcd_stout_force", "lqcd_deo_apply_mrhs_layout",
-    "lqcd_selftest_stage_wait", "lqcd_inject_alloc_failure", "lqcd_bounds_errors",
+    "lqcd_selftest_stage_wait", "lqcd_selftest_resident_wait", "lqcd_inject_alloc_failure", "lqcd_bounds_errors",
     "lqcd_shard_create", "lqcd_shard_geometry", "lqcd_shard_links_upload", "lqcd_shard_deo_apply",
     "lqcd_shard_exchange", "lqcd_shard_cg_solve", "lqcd_deo_tuned_config",
     "lqcd_measure_fma_rates", "lqcd_deo_apply_h16",
@@ -162,6 +162,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
         "lqcd_deo_apply_mrhs_layout": (ctypes.c_int, [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                       vp, vp, vp]),
         "lqcd_selftest_stage_wait": (ctypes.c_int, [vp, ctypes.c_double]),
+        "lqcd_selftest_resident_wait": (ctypes.c_int, [vp, ctypes.c_double]),
         "lqcd_inject_alloc_failure": (None, [ctypes.c_long]),
         "lqcd_bounds_errors": (ctypes.c_int, [ctypes.POINTER(ctypes.c_uint)]),
         "lqcd_stout_smear": (ctypes.c_int, [vp, ctypes.c_double, ctypes.c_int]),
@@ -353,6 +354,10 @@ class Context:
         """Run the bounded-wait self-test (lqcd_selftest_stage_wait); raises
         LqcdError with status LQCD_ETIMEOUT when the wait ran out as designed."""
         check(self.lib.lqcd_selftest_stage_wait(self.h, float(limit_s)))
+
+    def selftest_resident_wait(self, limit_s: float = 0.05):
+        """The same for the waits of the resident iteration (lqcd_selftest_resident_wait)."""
+        check(self.lib.lqcd_selftest_resident_wait(self.h, float(limit_s)))
 
     def stout_smear(self, rho: float, levels: int):
         """Smear the links `levels` times (lqcd_stout_smear)."""
