@@ -135,20 +135,24 @@ __device__ __forceinline__ void red_add(unsigned *p, unsigned n)
     asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(n) : "memory");
 }
 
-// Until *p has reached n, or the time limit has passed (false).
+// Until *p has reached n, or the time limit has passed (false).  The count is
+// read once more after that: a block that was preempted may find it complete.
 template <bool ACQ>
 __device__ __forceinline__ bool poll_count(const unsigned *p, unsigned n, uint64_t limit_ns)
 {
-    uint64_t t0 = 0;
-    for (unsigned k = 1;; ++k) {
+    auto reached = [=]() -> bool {
         unsigned v;
         if (ACQ) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
         else asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-        if ((int)(v - n) >= 0) return true;
+        return (int)(v - n) >= 0;
+    };
+    uint64_t t0 = 0;
+    for (unsigned k = 1;; ++k) {
+        if (reached()) return true;
         if ((k & 63u) == 0u) {
             const uint64_t t = globaltimer_ns();
             if (t0 == 0) t0 = t;
-            if (t - t0 > limit_ns) return false;
+            if (t - t0 > limit_ns) return reached();
         }
     }
 }
@@ -192,7 +196,8 @@ __device__ __noinline__ double res_warp_total(ResShared &sh, const ulonglong2 *X
                     const uint64_t t = globaltimer_ns();
                     if (t0 == 0) t0 = t;
                     if (t - t0 > limit_ns) {
-                        sh.dead = 1;
+                        v[k] = xch_get(p + k);
+                        if (!xch_ok(v[k], tag)) sh.dead = 1;
                         break;
                     }
                 }
