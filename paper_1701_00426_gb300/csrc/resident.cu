@@ -224,11 +224,14 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     LQCD_CUDA(cudaEventCreateWithFlags(&ev[0], cudaEventDisableTiming));
     LQCD_CUDA(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
     auto enqueue = [&](int sl) -> cudaError_t {
-        // a fresh range of tags for every launch, 0 left out (the cleared buffer)
-        if (c->res_tag > 0xFFFF0000u) c->res_tag = 0;
+        // a fresh range of tags for every launch, 0 left out (the cleared buffer);
+        // when they start again, no sum of the first round may be left
+        const bool wrap = c->res_tag > 0xFFFF0000u;
+        if (wrap) c->res_tag = 0;
         R.tag0 = c->res_tag + 1;
         c->res_tag += (uint32_t)R.steps;
-        cudaError_t e = cudaMemsetAsync(c->res_xch.ptr, 0, (size_t)B.njobs * kResWords * sizeof(unsigned), s);
+        cudaError_t e = cudaMemsetAsync(c->res_xch.ptr, 0,
+                                        wrap ? c->res_xch.bytes : (size_t)B.njobs * kResWords * sizeof(unsigned), s);
         if (e != cudaSuccess) return e;
         res_launch<NJ>(R, vp, lf, blocks, smem, s);
         e = cudaGetLastError();
