@@ -195,27 +195,23 @@ __device__ __forceinline__ int step_delta(const LinkGeo &g, const int (&x)[4], i
 
 // Links on their way from L2 to a thread: D slots of nine components per thread
 // of the block, filled with cp.async.  A thread reads only what it copied.
-template <class T>
 struct LinkRing {
-    static constexpr int D = sizeof(T) == 4 ? 4 : 2;
-    static constexpr bool keep = sizeof(T) == 4;   // one more slot, for the link that every side takes
-    typename Vec2T<T>::t e[D + (keep ? 1 : 0)][9][kGaugeThreads];
+    static constexpr int D = 4;
+    float2 e[D + 1][9][kGaugeThreads];   // slot D: the link that every side takes
 };
 
 // U_dir at a site into slot (one group; an empty one if !live)
-template <class T>
-__device__ __forceinline__ void ring_fetch(LinkRing<T> &R, int slot, const typename Vec2T<T>::t *__restrict__ L, int dir,
-                                           SiteIdx s, int Vh, bool live = true)
+__device__ __forceinline__ void ring_fetch(LinkRing &R, int slot, const float2 *__restrict__ L, int dir, SiteIdx s, int Vh,
+                                           bool live = true)
 {
-    using V = typename Vec2T<T>::t;
     if (live) {
         const unsigned off = ((unsigned)((dir * 2 + s.par) * 9) * (unsigned)Vh + (unsigned)s.idx);
         const unsigned d = (unsigned)__cvta_generic_to_shared(&R.e[slot][0][threadIdx.x]);
 #pragma unroll
         for (int c = 0; c < 9; ++c)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d + c * (unsigned)(kGaugeThreads * sizeof(V))),
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d + c * (unsigned)(kGaugeThreads * sizeof(float2))),
                          "l"(L + (size_t)c * Vh + off), "n"
-                         (sizeof(V))
+                         (sizeof(float2))
                          : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -223,13 +219,12 @@ __device__ __forceinline__ void ring_fetch(LinkRing<T> &R, int slot, const typen
 
 // The link in a slot, or its conjugate transpose (read transposed, imaginary
 // parts negated).
-template <class T>
-__device__ __forceinline__ void ring_read(const LinkRing<T> &R, int slot, bool dag, Mat3<T> &U)
+__device__ __forceinline__ void ring_read(const LinkRing &R, int slot, bool dag, Mat3<float> &U)
 {
     const int row = dag ? 1 : 3, col = dag ? 3 : 1;
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
-        const typename Vec2T<T>::t v = R.e[slot][(c / 3) * row + (c % 3) * col][threadIdx.x];
+        const float2 v = R.e[slot][(c / 3) * row + (c % 3) * col][threadIdx.x];
         U.e[c] = {v.x, dag ? -v.y : v.y};
     }
 }
@@ -255,11 +250,11 @@ __device__ __forceinline__ void coords_of(const LinkGeo &g, int P, int i, int (&
 // Twelve links of a side come through the ring in the order of their use, D - 1
 // links ahead, across sides.
 constexpr int kSideLinks = 12;
-template <class T>
-__device__ __forceinline__ void staple_sum_dev(const LinkGeo &g, const typename Vec2T<T>::t *__restrict__ L,
-                                               LinkRing<T> &R, const int (&x)[4], int P, int i, int mu, Mat3<T> &A)
+__device__ __forceinline__ void staple_sum_f32(const LinkGeo &g, const float2 *__restrict__ L, LinkRing &R,
+                                               const int (&x)[4], int P, int i, int mu, Mat3<float> &A)
 {
-    constexpr int D = LinkRing<T>::D;
+    using T = float;
+    constexpr int D = LinkRing::D;
     const int Vh = g.Vh;
 #pragma unroll
     for (int k = 0; k < 9; ++k) A.e[k] = {T(0), T(0)};
@@ -286,12 +281,12 @@ __device__ __forceinline__ void staple_sum_dev(const LinkGeo &g, const typename 
             case 10: s = at(d1, 1); break;
             default: dir = nu; s = up ? SiteIdx{P, i} : at(d1, 1); break;
         }
-        ring_fetch<T>(R, slot, L, dir, s, Vh, live);
+        ring_fetch(R, slot, L, dir, s, Vh, live);
     };
     int w = mu == 0 ? 2 : 0;
     int d1 = step_delta(g, x, w >> 1, -1);
     const SiteIdx b1 = at(db1, 1);
-    if (LinkRing<T>::keep) ring_fetch<T>(R, D, L, mu, b1, Vh);   // U_mu(x - mu)
+    ring_fetch(R, D, L, mu, b1, Vh);   // U_mu(x - mu)
 #pragma unroll
     for (int k = 0; k < D - 1; ++k) fetch(k, k, w >> 1, false, d1, 0, true);
 #pragma unroll 1
@@ -308,7 +303,7 @@ __device__ __forceinline__ void staple_sum_dev(const LinkGeo &g, const typename 
         // link k into U, and the one D - 1 further on into the slot of link k - 1
         auto take = [&](int k, bool dag, Mat3<T> &U) {
             asm volatile("cp.async.wait_group %0;" ::"n"(D - 2) : "memory");
-            ring_read<T>(R, k % D, dag, U);
+            ring_read(R, k % D, dag, U);
             const int f = k + D - 1;
             if (f < kSideLinks) fetch(f % D, f, nu, up, d1, d2, true);
             else fetch(f % D, f - kSideLinks, nn, un, dn, 0, wn < 8);
@@ -324,8 +319,7 @@ __device__ __forceinline__ void staple_sum_dev(const LinkGeo &g, const typename 
         mat_mul(Q, t1, t2);
         take(3, up, t1);
         mat_mul(t2, t1, W);
-        if (LinkRing<T>::keep) ring_read<T>(R, D, false, t1);
-        else load_link_soa<T>(L, mu, b1.par, b1.idx, Vh, t1);
+        ring_read(R, D, false, t1);
         mat_mul(W, t1, t2);
         mat_axpy(c1, t2, A);
         // W = c0 Q + c1 (a' + c'), multiplied by E below
@@ -377,8 +371,7 @@ __device__ __forceinline__ void dm_load(const float4 *__restrict__ L, int mu, in
     }
 }
 
-// c = a b (dg = false) or a b^dag (dg = true)
-template <bool dg>
+// c = a b
 __device__ __forceinline__ void dm_mul(const DM3 &a, const DM3 &b, DM3 &c)
 {
 #pragma unroll
@@ -389,16 +382,15 @@ __device__ __forceinline__ void dm_mul(const DM3 &a, const DM3 &b, DM3 &c)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const DC x = a.e[i * 3 + k];
-                const DC y = dg ? b.e[j * 3 + k] : b.e[k * 3 + j];
-                const float2 yi = dg ? df_neg(y.im) : y.im;  // conj for the dagger
+                const DC y = b.e[k * 3 + j];
                 if (k == 0) {
                     acc_first(re, x.re.x, x.re.y, y.re.x, y.re.y);
-                    acc_first(im, x.re.x, x.re.y, yi.x, yi.y);
+                    acc_first(im, x.re.x, x.re.y, y.im.x, y.im.y);
                 } else {
                     acc_prod(re, x.re.x, x.re.y, y.re.x, y.re.y);
-                    acc_prod(im, x.re.x, x.re.y, yi.x, yi.y);
+                    acc_prod(im, x.re.x, x.re.y, y.im.x, y.im.y);
                 }
-                acc_prod(re, -x.im.x, -x.im.y, yi.x, yi.y);
+                acc_prod(re, -x.im.x, -x.im.y, y.im.x, y.im.y);
                 acc_prod(im, x.im.x, x.im.y, y.re.x, y.re.y);
             }
             c.e[i * 3 + j].re = acc_result(re);
@@ -460,101 +452,6 @@ __device__ __forceinline__ void mm_inplace(Mat3<R> &a, const Mat3<R> &b)
     }
 }
 
-// A += s t (s a df64 scalar)
-__device__ __forceinline__ void dm_axpy(float2 s, const DM3 &t, DM3 &A)
-{
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        A.e[q].re = df_fma(s, t.e[q].re, A.e[q].re);
-        A.e[q].im = df_fma(s, t.e[q].im, A.e[q].im);
-    }
-}
-
-__device__ __forceinline__ void dm_at(const LinkGeo &g, const float4 *L, const int (&x)[4], const int (&d)[4], int dir,
-                                      DM3 &U)
-{
-    int par, idx;
-    site_of(g, x, d[0], d[1], d[2], d[3], par, idx);
-    dm_load(L, dir, par, idx, g.Vh, U);
-}
-
-// Staple paths as step tables, all starting at x + mu and ending at x
-// (direction 0 = mu, 1 = nu; the sign of a nu step is multiplied by s):
-//   plaquette      nu, -mu, -nu                   (coefficient c0)
-//   rectangle (a)  mu, nu, -mu, -mu, -nu          (c1)
-//   rectangle (b)  nu, -mu, -mu, -nu, mu          (c1)
-//   rectangle (c)  nu, nu, -mu, -nu, -nu          (c1)
-// One loop with a single product site keeps the double-float code small
-// enough for the instruction cache: with the staple chains unrolled (78
-// products of ~1400 instructions) the kernel stalled on instruction fetch
-// (46 ns/site at 32^4, 25.6 with the loop, 84 products).  In FP32 and native
-// FP64 a product is ~110 instructions and the shared-prefix form of
-// staple_sum_dev (67 products) is faster (2.7 against 3.2 ns/site in FP32).
-__device__ __forceinline__ int path_len(int p) { return p == 0 ? 3 : 5; }
-__device__ __forceinline__ int path_dir(int p, int k)
-{
-    // bit k of the mask: 1 = nu step
-    const unsigned m = p == 0 ? 0x5u : (p == 1 ? 0x12u : (p == 2 ? 0x9u : 0x1Bu));
-    return (int)((m >> k) & 1u);
-}
-__device__ __forceinline__ int path_sgn(int p, int k)
-{
-    // bit k of the mask: 1 = positive step
-    const unsigned m = p == 0 ? 0x1u : (p == 1 ? 0x3u : (p == 2 ? 0x11u : 0x3u));
-    return ((m >> k) & 1u) ? 1 : -1;
-}
-
-__device__ void staple_sum_df_paths(const LinkGeo &g, const float4 *L, const int (&x)[4], int mu, DM3 &A)
-{
-#pragma unroll
-    for (int q = 0; q < 9; ++q) A.e[q].re = A.e[q].im = make_float2(0.f, 0.f);
-    const float2 c0 = make_float2((float)kSymC0, (float)(kSymC0 - (double)(float)kSymC0));
-    const float2 c1 = make_float2((float)kSymC1, (float)(kSymC1 - (double)(float)kSymC1));
-#pragma unroll 1
-    for (int nu = 0; nu < 4; ++nu) {
-        if (nu == mu) continue;
-#pragma unroll 1
-        for (int s = -1; s <= 1; s += 2) {
-#pragma unroll 1
-            for (int p = 0; p < 4; ++p) {
-                int d[4] = {0, 0, 0, 0};
-                d[mu] = 1;
-                DM3 M, u, T;
-                const int len = path_len(p);
-#pragma unroll 1
-                for (int k = 0; k < len; ++k) {
-                    const int isnu = path_dir(p, k);
-                    const int D = isnu ? nu : mu;
-                    const int sg = path_sgn(p, k) * (isnu ? s : 1);
-                    if (sg < 0) d[D] -= 1;
-                    dm_at(g, L, x, d, D, u);
-                    if (sg > 0) d[D] += 1;
-                    if (sg < 0) {
-#pragma unroll
-                        for (int i = 0; i < 3; ++i)
-#pragma unroll
-                            for (int j = 0; j < 3; ++j) {
-                                if (j <= i) continue;
-                                const DC a = u.e[i * 3 + j], b = u.e[j * 3 + i];
-                                u.e[i * 3 + j] = {b.re, df_neg(b.im)};
-                                u.e[j * 3 + i] = {a.re, df_neg(a.im)};
-                            }
-#pragma unroll
-                        for (int i = 0; i < 3; ++i) u.e[i * 4].im = df_neg(u.e[i * 4].im);
-                    }
-                    if (k == 0) {
-                        M = u;
-                    } else {
-                        dm_mul<false>(M, u, T);
-                        M = T;
-                    }
-                }
-                dm_axpy(p == 0 ? c0 : c1, M, A);
-            }
-        }
-    }
-}
-
 // H -= eps F at one link from M = U A (FP64, about 20 operations): F = traceless
 // part of -(i beta / 6)(M - M^dag), 8 reals with stride Vh.
 __device__ __forceinline__ void gauge_kick(const double (&mre)[9], const double (&mim)[9], double *h, int Vh,
@@ -573,33 +470,6 @@ __device__ __forceinline__ void gauge_kick(const double (&mre)[9], const double 
     f[7] = beta6 * (mre[7] - mre[5]);
 #pragma unroll
     for (int k = 0; k < 8; ++k) h[(size_t)k * Vh] = fma(-eps, f[k], h[(size_t)k * Vh]);
-}
-
-// The path form, for a device without room for the stored staples.
-// H_mu(x) -= eps F_mu(x) with the staple sum and U A in double-float; F
-// and the update itself in native FP64 (about 20 operations per link).
-__global__ void __launch_bounds__(kGaugeThreads)
-    k_gauge_mom_update_df(LinkGeo g, const float4 *__restrict__ L, double *__restrict__ mom, double beta6, double eps)
-{
-    const int Vh = g.Vh;
-    const long t = blockIdx.x * (long)kGaugeThreads + threadIdx.x;
-    if (t >= 8L * Vh) return;
-    const int i = (int)(t % Vh);
-    const int mp = (int)(t / Vh);
-    const int mu = mp >> 1, P = mp & 1;
-    int x[4];
-    coords_of(g, P, i, x);
-    DM3 A, U, M;
-    staple_sum_df_paths(g, L, x, mu, A);
-    dm_load(L, mu, P, i, Vh, U);
-    dm_mul<false>(U, A, M);
-    double mre[9], mim[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-        mre[q] = df_to_f64(M.e[q].re);
-        mim[q] = df_to_f64(M.e[q].im);
-    }
-    gauge_kick(mre, mim, mom + (size_t)(mp * 8) * Vh + i, Vh, beta6, eps);
 }
 
 // ------------------------------------------------------------------ scalar arithmetic
@@ -624,7 +494,7 @@ template <> __device__ __forceinline__ float2 r_of<float2>(double v) { return f6
 __device__ __forceinline__ double r_double(double a) { return a; }
 __device__ __forceinline__ double r_double(float2 a) { return df_to_f64(a); }
 __device__ __forceinline__ void mm(const Mat3<double> &a, const Mat3<double> &b, Mat3<double> &c) { mat_mul(a, b, c); }
-__device__ __forceinline__ void mm(const DM3 &a, const DM3 &b, DM3 &c) { dm_mul<false>(a, b, c); }
+__device__ __forceinline__ void mm(const DM3 &a, const DM3 &b, DM3 &c) { dm_mul(a, b, c); }
 
 // 1 / n!, rounded to FP64 and split into double-float pairs
 constexpr int kExpDegMax = 20;
@@ -827,7 +697,7 @@ __global__ void __launch_bounds__(kGaugeThreads)
     DM3 E, U, W;
     exp_herm(herm_from<float2>(h, eps), E);
     dm_load(Ldf, mp >> 1, mp & 1, i, Vh, U);
-    dm_mul<false>(E, U, W);
+    dm_mul(E, U, W);
     double2 *pn = nat + (size_t)(mp * 9) * Vh + i;
     float4 *pd = Ldf + (size_t)(mp * 9) * Vh + i;
 #pragma unroll
@@ -856,14 +726,11 @@ __global__ void __launch_bounds__(kGaugeThreads)
 // links' 24 sides 120: 160 products per site with U A, where the separate
 // paths take 340, and 5 neighbour sites per plane instead of 17.  Bound by the
 // FP32 pipes (double-float) or the FP64 pipe (native).  Momentum update,
-// paths -> stored staples: double-float 1542 -> 785 us at 16^4, 7437 -> 3828 at
-// 24^4, 23.2 -> 15.5 ms at 32^4; native 3750 -> 2543 us at 16^4.
+// separate paths -> stored staples: double-float 1542 -> 645 us at 16^4, 7.44 ->
+// 3.06 ms at 24^4, 23.2 -> 11.8 at 32^4; native 3750 -> 2207 us at 16^4.
 // The staples of np of the six planes at a time are kept (576 bytes per site
 // and plane); the force is linear in A, so planes may be added one pass after
-// another.  Four blocks per SM with two matrices of a thread in shared memory
-// (128 registers); with all in registers (255, two blocks) the update takes
-// 1033 us at 16^4, with three or five blocks 768 and 838 (17.0 and 15.8 ms at
-// 32^4).
+// another.
 template <class R> struct SideT;
 template <> struct SideT<float2> { using t = float4; };
 template <> struct SideT<double> { using t = double2; };
@@ -973,6 +840,42 @@ __device__ __forceinline__ Cplx<double> side_elem(const double2 &v, bool dag)
     return {v.x, flip_sign(v.y, dag ? 0x80000000u : 0u)};
 }
 
+// M <- M^dag
+template <class R>
+__device__ __forceinline__ void conj_transpose(Mat3<R> &M)
+{
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = i; j < 3; ++j) {
+            const Cplx<R> a = M.e[i * 3 + j], b = M.e[j * 3 + i];
+            M.e[i * 3 + j] = {b.re, r_neg(b.im)};
+            M.e[j * 3 + i] = {a.re, r_neg(a.im)};
+        }
+}
+
+// up_mn(y) or, with down, down_mn(y + n): the products of k_gauge_sides in their order,
+// so the same bits as the stored ones.
+template <class R>
+__device__ __forceinline__ void plaquette_side(const LinkGeo &g, const typename SideT<R>::t *__restrict__ L,
+                                               const int (&y)[4], bool down, int m, int n, Mat3<R> &M)
+{
+    const int p = down ? m : n, q = down ? n : m;
+    const SiteIdx s0 = site_step(g, y, p, 0);
+    Mat3<R> u;
+    load_side(L, p, s0, g.Vh, false, M);
+    load_side(L, q, site_step(g, y, p, 1), g.Vh, false, u);
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        mm_inplace(M, u);   // C = U_p(y) U_q(y+p); C U_p(y+q)^dag or U_q(y)^dag C
+        if (k == 0 && !down) load_side(L, p, site_step(g, y, q, 1), g.Vh, true, u);
+        if (k == 0 && down) {
+            u = M;
+            load_side(L, q, s0, g.Vh, true, M);
+        }
+    }
+}
+
 // Stored staples of the planes pr: thread = (ordered pair (p, q), parity, site);
 // C = U_p(x) U_q(x+p) gives up_qp(x) = C U_p(x+q)^dag and
 // down_pq(x+q) = U_q(x)^dag C.  One product in a loop: unrolled, the
@@ -1020,8 +923,12 @@ __global__ void __launch_bounds__(kGaugeThreads, 4)
 // 784 -> 645 us, 24^4 3.81 -> 3.06 ms, 32^4 15.5 -> 11.8, 8^4 102 -> 91.  Three and
 // five blocks per SM: 689 and 681 at 16^4.  Native FP64, where the signs of the
 // conjugates moved to the integer pipe: 16^4 2543 -> 2207 us.
-template <class R>
-__global__ void __launch_bounds__(kGaugeThreads, 4)
+// STORED = false, for a device without room for the staples: each thread forms
+// the three staples of a side when it needs them, 67 products per link, with the
+// same bits.  8^4 131 us (99 stored), 16^4 1059 (645), 24^4 5.69 ms (3.06); native
+// 307, 3765, 18.4 ms.
+template <class R, bool STORED>
+__global__ void __launch_bounds__(kGaugeThreads, STORED ? 4 : 2)
     k_gauge_mom_sides(LinkGeo g, PlaneRange pr, const typename SideT<R>::t *__restrict__ L,
                       const typename SideT<R>::t *__restrict__ F, double *__restrict__ mom, double beta6, double eps)
 {
@@ -1082,16 +989,38 @@ __global__ void __launch_bounds__(kGaugeThreads, 4)
         for (int k = 0; k < 5; ++k) {
             // B = X Y; A += B (Z' - 20 Z); B = X' Y; B += X Y'; A += B Z
             const bool zz = k == 1 || k == 4;
-            load_side(k == 3 ? F : L, k == 3 ? ky : (zz ? nu : mu), zz ? sz : sy, Vh, zz ? lower == 0 : true, u);
+            Mat3<R> z;   // Z'; X', Y' and Z' where they are not stored
+            if constexpr (!STORED) {
+                if (k >= 1 && k <= 3) {
+                    // X' = up_{nu mu}(x+mu(-nu)), Y' = up_{mu nu}(x+nu) or down_{mu nu}(x-nu), Z' = down_{nu mu}(x(-nu))
+                    const int dm = k == 2 ? 1 : (k == 3 ? 0 : -1);
+                    const int dn = k == 3 ? (lower ? -2 : 1) : -lower;
+                    int y[4];
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) y[d] = wrap(x[d] + (d == mu ? dm : 0) + (d == nu ? dn : 0), g.N[d]);
+                    plaquette_side(g, L, y, k == 1 || (k == 3 && lower), k == 3 ? mu : nu, k == 3 ? nu : mu, z);
+                    if (k == 3 || (k == 1) == (lower == 0)) conj_transpose(z);
+                    if (k == 2) {
+#pragma unroll
+                        for (int q = 0; q < 9; ++q) put_elem(B, q, z.e[q]);
+                    }
+                }
+            }
+            if constexpr (STORED) {
+                load_side(k == 3 ? F : L, k == 3 ? ky : (zz ? nu : mu), zz ? sz : sy, Vh, zz ? lower == 0 : true, u);
+                if (k == 1) load_side(F, kx + 1, sz, Vh, lower == 0, z);
+            } else {
+                if (k == 3) u = z;
+                else load_side(L, zz ? nu : mu, zz ? sz : sy, Vh, zz ? lower == 0 : true, u);
+            }
             if (k == 1) {
-                Mat3<R> z;
-                load_side(F, kx + 1, sz, Vh, lower == 0, z);
 #pragma unroll
                 for (int q = 0; q < 9; ++q)
                     u.e[q] = {minus20(z.e[q].re, u.e[q].re), minus20(z.e[q].im, u.e[q].im)};
             }
             T *D = zz ? A : B;
-            product(zz ? nullptr : (k == 2 ? F : L), k == 2 ? kx : nu, sx, !zz && lower != 0, D, k == 3 || (zz && any), D);
+            const bool left = zz || (!STORED && k == 2);   // the left factor is B
+            product(left ? nullptr : (k == 2 ? F : L), k == 2 ? kx : nu, sx, !left && lower != 0, D, k == 3 || (zz && any), D);
             any |= zz;
         }
     }
@@ -1152,10 +1081,10 @@ __device__ __forceinline__ const T *mom_ptr(const T *m, int mu, int P, int Vh)
 // 636; some links through the ring and some straight: 619 to 679, slower at
 // 32^4; bodies of their own for s = -1 and s = +1, without selections, outgrow the
 // instruction cache: 667.
-template <class T>
-__global__ void __launch_bounds__(kGaugeThreads, sizeof(T) == 4 ? 3 : 2)
-    k_gauge_mom_update(LinkGeo g, const typename Vec2T<T>::t *__restrict__ L, T *__restrict__ mom, T beta6, T eps)
+__global__ void __launch_bounds__(kGaugeThreads, 3)
+    k_gauge_mom_update_f32(LinkGeo g, const float2 *__restrict__ L, float *__restrict__ mom, float beta6, float eps)
 {
+    using T = float;
     static_assert(kGaugeThreads == 128, "four directions of 32 sites");
     const int Vh = g.Vh, nt = (Vh + 31) / 32;
     const int P = (int)blockIdx.x / nt, i = ((int)blockIdx.x - P * nt) * 32 + ((int)threadIdx.x & 31);
@@ -1164,8 +1093,8 @@ __global__ void __launch_bounds__(kGaugeThreads, sizeof(T) == 4 ? 3 : 2)
     int x[4];
     coords_of(g, P, i, x);
     Mat3<T> A, U, M;
-    __shared__ LinkRing<T> ring;
-    staple_sum_dev<T>(g, L, ring, x, P, i, mu, A);
+    __shared__ LinkRing ring;
+    staple_sum_f32(g, L, ring, x, P, i, mu, A);
     load_link_soa<T>(L, mu, P, i, Vh, U);
     mat_mul(U, A, M);
     // F = -(i beta/6)(M - M^dag): F_ij = (beta/6) * (i (conj(M_ji) - M_ij))
@@ -1983,58 +1912,63 @@ static int check_md(lqcd_ctx *c, int prec)
     return LQCD_OK;
 }
 
-// Planes whose staples are stored at a time: as many of 6, 3, 2, 1 as fit the
-// scratch limit (all six up to 24^4, three at 32^4, one at 48^4: 3.1 GB there).
-// 0: no room even for one plane.
+// Planes of one pass of the FP64 momentum update: as many of 6, 3, 2, 1 as keep the
+// stored staples within kSidesLimit (all six up to 24^4, three at 32^4, two up to
+// 36^4, one beyond: 3.1 GB at 48^4).  The passes group the sum into H, so their number depends on
+// the lattice alone, and the bits do not depend on how much memory is free.
 constexpr size_t kSidesLimit = (size_t)2 << 30;
 
-static int sides_planes(lqcd_ctx *c)
+static size_t plane_bytes(const lqcd_ctx *c) { return (size_t)1152 * c->Vh; }
+
+static int sides_planes(const lqcd_ctx *c)
 {
-    const size_t plane = (size_t)1152 * c->Vh;
     int np = 6;
-    while (np > 1 && np * plane > kSidesLimit) np = np == 6 ? 3 : np - 1;
-    for (; np >= 1; np = np == 6 ? 3 : np - 1) {
-        if (c->md_sides.bytes >= np * plane || c->md_sides.ensure(np * plane) == LQCD_OK) return np;
-        set_error("");
-    }
-    return 0;
+    while (np > 1 && np * plane_bytes(c) > kSidesLimit) np = np == 6 ? 3 : np - 1;
+    return np;
+}
+
+// Room for the stored staples; false: the kernel that forms them itself runs.
+// Asked once per call, before its first launch.
+static bool sides_room(lqcd_ctx *c, int prec)
+{
+    if (prec == LQCD_PREC_FP32) return false;
+    if (c->md_sides.ensure(sides_planes(c) * plane_bytes(c)) == LQCD_OK) return true;
+    set_error("");
+    return false;
 }
 
 template <class R>
-static void launch_mom_sides(lqcd_ctx *c, const typename SideT<R>::t *L, int np, double beta, double eps)
+static void launch_mom_sides(lqcd_ctx *c, const typename SideT<R>::t *L, bool stored, double beta, double eps)
 {
     const LinkGeo g = link_geo(c);
+    const int np = sides_planes(c);
     typename SideT<R>::t *F = c->md_sides.as<typename SideT<R>::t>();
+    double *mom = c->mom64.as<double>();
     const unsigned nt = (unsigned)(2 * ((c->Vh + 31) / 32));
     for (int p0 = 0; p0 < 6; p0 += np) {
         const PlaneRange pr = {p0, np};
-        k_gauge_sides<R><<<nblocks(4L * np * (long)c->Vh, kGaugeThreads), kGaugeThreads, 0, c->stream>>>(g, pr, L, F);
-        k_gauge_mom_sides<R><<<nt, kGaugeThreads, 0, c->stream>>>(g, pr, L, F, c->mom64.as<double>(), beta / 6.0, eps);
-        c->launches += 2;
+        if (stored) {
+            k_gauge_sides<R><<<nblocks(4L * np * (long)c->Vh, kGaugeThreads), kGaugeThreads, 0, c->stream>>>(g, pr, L, F);
+            k_gauge_mom_sides<R, true><<<nt, kGaugeThreads, 0, c->stream>>>(g, pr, L, F, mom, beta / 6.0, eps);
+        } else {
+            k_gauge_mom_sides<R, false><<<nt, kGaugeThreads, 0, c->stream>>>(g, pr, L, nullptr, mom, beta / 6.0, eps);
+        }
+        c->launches += stored ? 2 : 1;
     }
 }
 
-static void launch_mom_update(lqcd_ctx *c, int prec, double beta, double eps)
+static void launch_mom_update(lqcd_ctx *c, int prec, bool stored, double beta, double eps)
 {
-    const LinkGeo g = link_geo(c);
-    const unsigned nb = nblocks(8L * (long)c->Vh, kGaugeThreads);
-    const unsigned nt = (unsigned)(2 * ((c->Vh + 31) / 32));
-    const int np = prec == LQCD_PREC_FP32 ? 0 : sides_planes(c);
-    if (np > 0) {
-        if (prec == LQCD_PREC_FP64) launch_mom_sides<float2>(c, c->lnk_df.as<float4>(), np, beta, eps);
-        else launch_mom_sides<double>(c, c->lnk_nat.as<double2>(), np, beta, eps);
-        return;
+    if (prec == LQCD_PREC_FP64) {
+        launch_mom_sides<float2>(c, c->lnk_df.as<float4>(), stored, beta, eps);
+    } else if (prec == LQCD_PREC_FP64_NATIVE) {
+        launch_mom_sides<double>(c, c->lnk_nat.as<double2>(), stored, beta, eps);
+    } else {
+        const unsigned nt = (unsigned)(2 * ((c->Vh + 31) / 32));
+        k_gauge_mom_update_f32<<<nt, kGaugeThreads, 0, c->stream>>>(link_geo(c), c->lnk_f18.as<float2>(),
+                                                                    c->mom32.as<float>(), (float)(beta / 6.0), (float)eps);
+        c->launches += 1;
     }
-    if (prec == LQCD_PREC_FP64)
-        k_gauge_mom_update_df<<<nb, kGaugeThreads, 0, c->stream>>>(g, c->lnk_df.as<float4>(), c->mom64.as<double>(),
-                                                                   beta / 6.0, eps);
-    else if (prec == LQCD_PREC_FP64_NATIVE)
-        k_gauge_mom_update<double><<<nt, kGaugeThreads, 0, c->stream>>>(g, c->lnk_nat.as<double2>(), c->mom64.as<double>(),
-                                                                        beta / 6.0, eps);
-    else
-        k_gauge_mom_update<float><<<nt, kGaugeThreads, 0, c->stream>>>(g, c->lnk_f18.as<float2>(), c->mom32.as<float>(),
-                                                                       (float)(beta / 6.0), (float)eps);
-    c->launches += 1;
 }
 
 static void launch_link_update(lqcd_ctx *c, int prec, double eps)
@@ -2174,7 +2108,7 @@ int lqcd_gauge_mom_update(lqcd_ctx *c, int prec, double beta, double eps)
     LQCD_ON_DEVICE(c->device);
     int st;
     if ((st = check_md(c, prec)) || (st = check_thin(c)) || (st = prepare(c, prec))) return st;
-    launch_mom_update(c, prec, beta, eps);
+    launch_mom_update(c, prec, sides_room(c, prec), beta, eps);
     LQCD_CUDA(cudaGetLastError());
     LQCD_CUDA(cudaStreamSynchronize(c->stream));
     return LQCD_OK;
@@ -2201,8 +2135,9 @@ int lqcd_gauge_md_steps(lqcd_ctx *c, int prec, double beta, double eps, int n_st
     int st;
     if ((st = check_md(c, prec)) || (st = check_thin(c)) || (st = prepare(c, prec))) return st;
     if (n_steps < 0) return fail(LQCD_EINVAL, "n_steps must be >= 0");
+    const bool stored = n_steps > 0 && sides_room(c, prec);
     for (int k = 0; k < n_steps; ++k) {
-        launch_mom_update(c, prec, beta, eps);
+        launch_mom_update(c, prec, stored, beta, eps);
         launch_link_update(c, prec, eps);
     }
     LQCD_CUDA(cudaGetLastError());
