@@ -145,8 +145,9 @@ const char *lqcd_last_error(void);
 
 /* Host-side fault injection for tests of the error paths: the k-th device
  * allocation from now (k >= 1) fails as an out-of-memory cudaMalloc would,
- * and the call that made it returns LQCD_ENOMEM; k <= 0 disarms.  Process
- * wide.  A failed lqcd_links_upload leaves the context without links
+ * and the call that made it returns LQCD_ENOMEM, unless it can do without (the
+ * scratch of the FP64 momentum update, which is also given back when another
+ * allocation of its context fails); k <= 0 disarms.  Process wide.  A failed lqcd_links_upload leaves the context without links
  * (LQCD_ESTATE until the next successful upload). */
 void lqcd_inject_alloc_failure(long k);
 
@@ -424,7 +425,8 @@ int lqcd_mom_download(lqcd_ctx *ctx, double *H, size_t n_doubles);
 /* H <- H - eps F(U) on every link.  The FP64 forms keep plaquette staples in
  * device scratch that stays with the context (6912 B per even site, bounded by
  * 2 GiB up to 36^4; 1152 B per even site on larger lattices); where it cannot be
- * had the update takes 1.5 to 1.9 times as long, with the same bits. */
+ * had the update takes 1.5 to 1.9 times as long, with the same bits.  It is given
+ * back when another allocation of a call on the context fails. */
 int lqcd_gauge_mom_update(lqcd_ctx *ctx, int prec, double beta, double eps);
 
 /* U <- exp(i eps H) U on every link (the exponential of the traceless

@@ -157,20 +157,36 @@ void prefault_host(void *p, size_t bytes)
     for (std::thread &t : th) t.join();
 }
 
+static thread_local const lqcd_ctx *t_context = nullptr;
+
+ContextScope::ContextScope(const lqcd_ctx *c) : up_(t_context) { t_context = c; }
+ContextScope::~ContextScope() { t_context = up_; }
+
+int device_of(const lqcd_ctx *c) { return c->device; }
+
 int DevBuf::ensure(size_t n)
 {
     if (n <= bytes && ptr) return LQCD_OK;
     release();
     if (n == 0) return LQCD_OK;
-    if (g_fail_alloc.load() > 0 && g_fail_alloc.fetch_sub(1) == 1)
-        return fail(LQCD_ENOMEM, "injected failure of a " + std::to_string(n) + "-byte device allocation");
-    cudaError_t e = cudaMalloc(&ptr, n);
-    if (e != cudaSuccess) {
+    const char *why = "cudaMalloc of ";
+    auto allocate = [&]() -> bool {
+        if (g_fail_alloc.load() > 0 && g_fail_alloc.fetch_sub(1) == 1) {
+            why = "injected failure of an allocation of ";
+            return false;
+        }
+        if (cudaMalloc(&ptr, n) == cudaSuccess) return true;
         ptr = nullptr;
-        bytes = 0;
         cudaGetLastError();
-        return fail(LQCD_ENOMEM, "cudaMalloc of " + std::to_string(n) + " bytes failed");
+        return false;
+    };
+    bool ok = allocate();
+    DevBuf *scratch = t_context ? &const_cast<lqcd_ctx *>(t_context)->md_sides : nullptr;
+    if (!ok && scratch && scratch->ptr && this != scratch) {
+        scratch->release();   // cudaFree waits for the kernels that use it
+        ok = allocate();
     }
+    if (!ok) return fail(LQCD_ENOMEM, why + std::to_string(n) + " bytes failed");
     bytes = n;
     return LQCD_OK;
 }
@@ -366,7 +382,7 @@ void lqcd_destroy(lqcd_ctx *c)
 int lqcd_set_opts(lqcd_ctx *c, const lqcd_opts *o)
 {
     if (!c || !o) return fail(LQCD_EINVAL, "NULL argument");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     int st = validate_opts(o);
     if (st) return st;
     c->opts = *o;
@@ -379,7 +395,7 @@ int lqcd_links_upload(lqcd_ctx *c, const double *links, size_t n)
 {
     NvtxRange nvtx_("lqcd_links_upload");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     c->graph.reset();
     return upload_links(c, links, n);
 }
@@ -387,7 +403,7 @@ int lqcd_links_upload(lqcd_ctx *c, const double *links, size_t n)
 int lqcd_links_download(lqcd_ctx *c, double *links, size_t n)
 {
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return download_links(c, links, n);
 }
 
@@ -395,7 +411,7 @@ int lqcd_deo_apply(lqcd_ctx *c, int out_parity, const void *in, void *out, int w
 {
     NvtxRange nvtx_("lqcd_deo_apply");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     if (where == 1) return deo_launch(c, out_parity, LQCD_PREC_FP64, 18, in, out, (cudaStream_t)stream ? (cudaStream_t)stream : c->stream);
     if (where != 0) return fail(LQCD_EINVAL, "where must be 0 (host) or 1 (device)");
     if (!in || !out) return fail(LQCD_EINVAL, "NULL spinor pointer");
@@ -420,7 +436,7 @@ int lqcd_deo_apply_ex(lqcd_ctx *c, int out_parity, int prec, int recon, const vo
 {
     NvtxRange nvtx_("lqcd_deo_apply_ex");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return deo_launch(c, out_parity, prec, recon, in, out, stream ? (cudaStream_t)stream : c->stream);
 }
 
@@ -428,21 +444,21 @@ int lqcd_deo_apply_mrhs(lqcd_ctx *c, int out_parity, int n_rhs, int recon, const
 {
     NvtxRange nvtx_("lqcd_deo_apply_mrhs");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return deo_mrhs_launch(c, out_parity, n_rhs, recon, in, out, stream ? (cudaStream_t)stream : c->stream);
 }
 
 int lqcd_selftest_stage_wait(lqcd_ctx *c, double limit_s)
 {
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return stage_wait_selftest(c, limit_s);
 }
 
 int lqcd_selftest_resident_wait(lqcd_ctx *c, double limit_s)
 {
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return resident_wait_selftest(c, limit_s);
 }
 
@@ -451,7 +467,7 @@ int lqcd_deo_apply_mrhs_layout(lqcd_ctx *c, int out_parity, int n_rhs, int recon
 {
     NvtxRange nvtx_("lqcd_deo_apply_mrhs_layout");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return deo_mrhs_launch(c, out_parity, n_rhs, recon, in, out, stream ? (cudaStream_t)stream : c->stream, layout);
 }
 
@@ -461,7 +477,7 @@ int lqcd_mscg_solve(lqcd_ctx *c, double mass, const double *shifts, int n_shift,
     NvtxRange nvtx_("lqcd_mscg_solve");
     const auto t0 = std::chrono::steady_clock::now();
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     if (!b || !x || !shifts) return fail(LQCD_EINVAL, "NULL argument");
     if (n_shift < 1 || n_shift > LQCD_MAX_SHIFTS) return fail(LQCD_EINVAL, "n_shift must be in 1..32");
     CallScope::declare(c->device, resident_sms(c));
@@ -489,7 +505,7 @@ int lqcd_mscg_solve_dev(lqcd_ctx *c, double mass, const double *shifts, int n_sh
 {
     NvtxRange nvtx_("lqcd_mscg_solve_dev");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     CallScope::declare(c->device, resident_sms(c));
     return mscg_solve_dev(c, mass, shifts, n_shift, tol, (const double2 *)b, (double2 *)x, info, (cudaStream_t)stream);
 }
@@ -498,7 +514,7 @@ int lqcd_profile_iteration(lqcd_ctx *c, double mass, const double *shifts, int n
                            int iters, double ms_out[4], double *n_active_avg)
 {
     if (!c || !ms_out || !n_active_avg) return fail(LQCD_EINVAL, "NULL argument");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return profile_iteration(c, mass, shifts, n_shift, tol, (const double2 *)b, iters, ms_out, n_active_avg);
 }
 
@@ -507,7 +523,7 @@ int lqcd_cg_solve_mrhs(lqcd_ctx *c, double mass, double sigma, int n_rhs, double
 {
     NvtxRange nvtx_("lqcd_cg_solve_mrhs");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     return cg_solve_mrhs(c, mass, sigma, n_rhs, tol, b, x, info);
 }
 
@@ -523,7 +539,7 @@ int lqcd_mscg_solve_packed(lqcd_ctx *const *ctxs, int n, const double *mass, con
         if (ctxs[i]->device != ctxs[0]->device)
             return fail(LQCD_EINVAL, "the contexts of a packed solve must live on one device");
     }
-    LQCD_ON_DEVICE(ctxs[0]->device);
+    LQCD_ON_DEVICE(ctxs[0]);
     return mscg_solve_packed(ctxs, n, mass, shifts, n_shift, tol, b, x, info);
 }
 

@@ -928,7 +928,7 @@ extern "C" int lqcd_deo_apply_h16(lqcd_ctx *c, int out_parity, const void *in, c
     using namespace lqcd;
     NvtxRange nvtx_("lqcd_deo_apply_h16");
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     if (int lr = links_ready(c)) return lr;
     if (out_parity != 0 && out_parity != 1) return fail(LQCD_EINVAL, "out_parity must be 0 or 1");
     if (!in || !in_norm || !out || !out_norm) return fail(LQCD_EINVAL, "NULL spinor pointer");

@@ -88,11 +88,29 @@ private:
     static CallScope *of(int dev);
 };
 
-// Every C entry point that receives a context (or a server) opens one of
-// these right after its NULL check.
-#define LQCD_ON_DEVICE(dev)                                                               \
-    ::lqcd::CallScope lqcd_call_scope_(dev);                                              \
-    ::lqcd::DeviceGuard lqcd_device_guard_(dev);                                          \
+// The context whose call runs on this thread.  When an allocation of the call
+// fails, scratch that the context keeps only to be faster (the stored staples) is
+// given back and the allocation tried again, so that what fitted without the
+// scratch still fits.
+struct ContextScope {
+    explicit ContextScope(const lqcd_ctx *c);
+    explicit ContextScope(int) : ContextScope(nullptr) {}   // a device without a context
+    ~ContextScope();
+    ContextScope(const ContextScope &) = delete;
+    ContextScope &operator=(const ContextScope &) = delete;
+
+private:
+    const lqcd_ctx *up_;
+};
+int device_of(const lqcd_ctx *c);
+inline int device_of(int dev) { return dev; }
+
+// Every C entry point that receives a context (or a server: its device) opens
+// one of these right after its NULL check.
+#define LQCD_ON_DEVICE(what)                                                              \
+    ::lqcd::ContextScope lqcd_context_scope_(what);                                       \
+    ::lqcd::CallScope lqcd_call_scope_(::lqcd::device_of(what));                          \
+    ::lqcd::DeviceGuard lqcd_device_guard_(::lqcd::device_of(what));                      \
     if (!lqcd_device_guard_.ok)                                                           \
         return ::lqcd::fail(LQCD_ECUDA, "cannot make the context's device current")
 

@@ -100,7 +100,7 @@ using namespace lqcd;
 extern "C" int lqcd_deo_apply_host_noalloc(lqcd_ctx *c, int out_parity, const double *in, double *out)
 {
     if (!c) return fail(LQCD_EINVAL, "NULL context");
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     if (!in || !out) return fail(LQCD_EINVAL, "NULL host buffer");
     if (out_parity != 0 && out_parity != 1) return fail(LQCD_EINVAL, "out_parity must be 0 or 1");
     if (int lr = links_ready(c)) return lr;

@@ -337,7 +337,7 @@ int lqcd_shard_links_upload(lqcd_ctx *c, const double *links, size_t n_doubles)
 {
     NvtxRange nvtx_("lqcd_shard_links_upload");
     if (int st = check_shard(c)) return st;
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     const long S = (long)c->gdims[0] * c->gdims[1] * c->gdims[2];
     const long Lt = c->gdims[3], V = S * Lt;
     if (!links || n_doubles != (size_t)(4 * V * 18))
@@ -363,7 +363,7 @@ int lqcd_shard_deo_apply(lqcd_ctx *c, int out_parity, const void *in, void *out,
 {
     NvtxRange nvtx_("lqcd_shard_deo_apply");
     if (int st = check_shard(c)) return st;
-    LQCD_ON_DEVICE(c->device);
+    LQCD_ON_DEVICE(c);
     if (int lr = links_ready(c)) return lr;
     if (out_parity != 0 && out_parity != 1) return fail(LQCD_EINVAL, "out_parity must be 0 or 1");
     if (!in || !out) return fail(LQCD_EINVAL, "NULL spinor pointer");
@@ -382,7 +382,7 @@ int lqcd_shard_exchange(lqcd_ctx *const *ctxs, int n, void *const *fields)
     NvtxRange nvtx_("lqcd_shard_exchange");
     if (int st = check_world(ctxs, n)) return st;
     if (!fields) return fail(LQCD_EINVAL, "NULL field array");
-    LQCD_ON_DEVICE(ctxs[0]->device);
+    LQCD_ON_DEVICE(ctxs[0]);
     return exchange_faces(ctxs, n, fields);
 }
 
@@ -609,7 +609,7 @@ extern "C" int lqcd_shard_cg_solve(lqcd_ctx *const *ctxs, int n, double mass, do
     if (int st = check_world(ctxs, n)) return st;
     if (!b || !x) return fail(LQCD_EINVAL, "NULL argument");
     if (!(tol > 0.0) || !std::isfinite(mass) || !(sigma >= 0.0)) return fail(LQCD_EINVAL, "bad mass, sigma or tol");
-    LQCD_ON_DEVICE(ctxs[0]->device);
+    LQCD_ON_DEVICE(ctxs[0]);
     if (info) memset(info, 0, sizeof *info);
     const auto t0 = std::chrono::steady_clock::now();
     const int st = shard_cg(ctxs, n, mass, sigma, tol, b, x, info);

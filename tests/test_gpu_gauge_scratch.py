@@ -65,3 +65,34 @@ def test_passes_over_the_planes(gpu, orc, prec, dims, planes):
         assert c.device_bytes() - before == planes * 1152 * (V // 2)
         got = c.mom_download() - spread(h)
     assert rel(got, spread(want)) <= (1e-12 if prec == 0 else 1e-13)
+
+
+def test_scratch_is_given_back_to_calls_that_need_memory(gpu):
+    """An allocation that fails while the context holds the scratch is tried again
+    without it; the momentum update then takes it anew, with the same bits."""
+    dims = (8, 8, 8, 8)
+    H = inputs.random_momenta(dims, seed=154)
+    b = inputs.gaussian_field(dims, k=9)
+    scratch = 6 * 1152 * 8 ** 4 // 2
+    with gpu.Context(dims) as c:
+        c.links_upload(inputs.random_links(dims, seed=154))
+        c.mom_upload(H)
+        c.gauge_mom_update(5.52, 0.03)
+        first = c.mom_download()
+        held = c.device_bytes()
+        gpu.inject_alloc_failure(1)
+        try:
+            x, info = c.mscg_solve(0.1, [1e-3], 1e-10, b)
+            assert c.device_bytes() < held                  # given back
+            gpu.inject_alloc_failure(1)
+            with pytest.raises(gpu.LqcdError) as e:         # nothing left to give
+                c.mscg_solve(0.1, inputs.log_shifts(8), 1e-10, b)
+            assert e.value.status == gpu.LQCD_ENOMEM
+        finally:
+            gpu.inject_alloc_failure(0)
+        assert max(info["true_resid"]) <= 1e-10
+        before = c.device_bytes()
+        c.mom_upload(H)
+        c.gauge_mom_update(5.52, 0.03)
+        assert c.device_bytes() == before + scratch
+        assert np.array_equal(c.mom_download(), first)
