@@ -364,7 +364,9 @@ int lqcd_rational_apply_dev(lqcd_ctx *ctx, double mass, double a0, const double 
  * multi-right-hand-side D_eo (each link loaded once per application for all
  * sources) with FP64 reliable updates; the solution and the true residual are
  * FP64.  b: host [n_rhs][Vh][3] complex128, x: same shape.  info: array of
- * n_rhs reports (or NULL).  Synchronous. */
+ * n_rhs reports (or NULL).  The device workspace stays with the context:
+ * 360 n_rhs + 48 bytes per even site for n_rhs a power of two, (n_rhs - 1) x 48
+ * less where there is no room for all residuals at once.  Synchronous. */
 int lqcd_cg_solve_mrhs(lqcd_ctx *ctx, double mass, double sigma, int n_rhs, double tol,
                        const double *b, double *x, lqcd_solve_info *info);
 

@@ -664,45 +664,54 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
     const int nt1 = (int)((Vh + kTile - 1) / kTile);
     const size_t npart = std::max((size_t)np * std::max(nb2, nbr), (size_t)nt1);
     if ((st = vec.ensure(5 * (size_t)n3 * np * sizeof(float2)))) return st;
-    if ((st = ieee.ensure((size_t)(n + 1) * n3 * sizeof(double2)))) return st;
+    // FP64 residuals that are formed together, with one synchronisation: all
+    // fields', or one where there is no room for them
+    int slots = n;
+    if ((st = ieee.ensure((size_t)(slots + 1) * n3 * sizeof(double2)))) {
+        if (n == 1) return st;
+        set_error("");
+        slots = 1;
+        if ((st = ieee.ensure((size_t)(slots + 1) * n3 * sizeof(double2)))) return st;
+    }
     if ((st = part.ensure((npart + 64) * sizeof(double)))) return st;
     if ((st = tick.ensure(64))) return st;
     if ((st = stb.ensure((size_t)np * sizeof(SolverState)))) return st;
     LQCD_CUDA(cudaMemsetAsync(tick.ptr, 0, 64, s));
     LQCD_CUDA(cudaMemsetAsync(vec.ptr, 0, 5 * (size_t)n3 * np * sizeof(float2), s));
     float2 *r = vec.as<float2>(), *p = r + n3 * np, *x = p + n3 * np, *q = x + n3 * np, *t = q + n3 * np;
-    double2 *rh = ieee.as<double2>(), *tn = rh + (size_t)n * n3;   // residuals of all fields, one temporary
+    double2 *rh = ieee.as<double2>(), *tn = rh + (size_t)slots * n3;   // residuals, one temporary
     SolverState *sts = stb.as<SolverState>();
     double *partd = part.as<double>(), *res = partd + npart;
     unsigned *tk = tick.as<unsigned>();
     const double2 *Lnat = c->lnk_nat.as<double2>();
     const unsigned nb3 = (unsigned)((n3 + 255) / 256);
     auto bj = [&](int j) { return b + (size_t)j * b_stride * n3; };
-    // FP64 true residuals of the fields listed, into rh and rr: all launches, then
-    // one synchronisation
-    auto true_res = [&](const std::vector<int> &js, std::vector<double> &rr) -> int {
-        for (int j : js) {
+    // FP64 true residuals of at most `slots` fields, into rh (in the order listed)
+    // and rr: all launches, then one synchronisation
+    auto true_res = [&](const int *js, int njs, std::vector<double> &rr) -> int {
+        for (int k = 0; k < njs; ++k) {
+            const int j = js[k];
             const double a = mass * mass + sigma[j];
             k_res_nat1_ext(c->g, Lnat, xh + (size_t)j * n3, tn, nt1, s);
-            k_res_nat2_ext(c->g, Lnat, tn, xh + (size_t)j * n3, bj(j), a, rh + (size_t)j * n3, partd, tk + 1, res + j, nt1,
+            k_res_nat2_ext(c->g, Lnat, tn, xh + (size_t)j * n3, bj(j), a, rh + (size_t)k * n3, partd, tk + 1, res + j, nt1,
                            s);
             LQCD_CUDA(cudaGetLastError());
             c->launches += 2;
         }
         LQCD_CUDA(cudaMemcpyAsync(c->h_pinned_d, res, kMaxRhs * sizeof(double), cudaMemcpyDeviceToHost, s));
         LQCD_CUDA(cudaStreamSynchronize(s));
-        for (int j : js) rr[j] = c->h_pinned_d[j];
+        for (int k = 0; k < njs; ++k) rr[js[k]] = c->h_pinned_d[js[k]];
         return LQCD_OK;
     };
     std::vector<double> b2(np, 0.0), scale(np, 1.0), target2(np, 0.0), rr(np, 0.0);
     std::vector<int> done(np, 1), rel(np, 0);
     const double delta = c->opts.delta_reliable;
-    // (re)start field j from the IEEE residual in rh: FP32 residual scaled to
-    // O(1) entries, x_lo = 0, p kept (rescaled) or set to r
-    auto restart = [&](int j, const SolverState *prev) -> int {
+    // (re)start field j from its IEEE residual: FP32 residual scaled to O(1)
+    // entries, x_lo = 0, p kept (rescaled) or set to r
+    auto restart = [&](int j, const double2 *resid, const SolverState *prev) -> int {
         const double old = scale[j];
         scale[j] = unit_scale_pub(rr[j], 6.0 * Vh);
-        k_col_from_ieee<<<nb3, 256, 0, s>>>(rh + (size_t)j * n3, r, n3, np, j, scale[j]);
+        k_col_from_ieee<<<nb3, 256, 0, s>>>(resid, r, n3, np, j, scale[j]);
         k_col_set<<<nb3, 256, 0, s>>>(x, nullptr, n3, np, j, 1);
         if (prev)
             k_col_scale<<<nb3, 256, 0, s>>>(p, n3, np, j, (float)(scale[j] / old));
@@ -730,12 +739,7 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
     idle.halt = HALT_CONVERGED;
     for (int j = 0; j < np; ++j) LQCD_CUDA(cudaMemcpyAsync(sts + j, &idle, sizeof idle, cudaMemcpyHostToDevice, s));
     // ||b_j||^2; the guess is zero, so b_j is also the first residual
-    std::vector<int> all_j(n);
-    for (int j = 0; j < n; ++j) {
-        all_j[j] = j;
-        k_norm2_ieee_ext(bj(j), (int)Vh, partd, tk + 1, nt1, res + j, s);
-        LQCD_CUDA(cudaMemcpyAsync(rh + (size_t)j * n3, bj(j), n3 * sizeof(double2), cudaMemcpyDeviceToDevice, s));
-    }
+    for (int j = 0; j < n; ++j) k_norm2_ieee_ext(bj(j), (int)Vh, partd, tk + 1, nt1, res + j, s);
     LQCD_CUDA(cudaGetLastError());
     c->launches += n;
     LQCD_CUDA(cudaMemcpyAsync(c->h_pinned_d, res, kMaxRhs * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -746,7 +750,7 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
         target2[j] = tol * tol * b2[j];
         if (rr[j] <= target2[j]) continue;   // b_j = 0, or tol >= 1: x_j = 0
         done[j] = 0;
-        if ((st = restart(j, nullptr))) return st;
+        if ((st = restart(j, bj(j), nullptr))) return st;
     }
     MrhsArgs A;
     memset(&A, 0, sizeof A);
@@ -826,8 +830,8 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
             c->launches += 1;
             js.push_back(j);
         }
-        if (rc == LQCD_OK && !js.empty()) rc = true_res(js, rr);
-        for (size_t k = 0; k < js.size() && rc == LQCD_OK; ++k) {
+        for (int k = 0; k < (int)js.size() && rc == LQCD_OK; ++k) {
+            if (k % slots == 0 && (rc = true_res(js.data() + k, std::min(slots, (int)js.size() - k), rr))) break;
             const int j = js[k];
             if (O[j].halt == HALT_MAXITER) { done[j] = 2; continue; }
             if (O[j].halt == HALT_RELIABLE) ++rel[j];
@@ -839,7 +843,7 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
                 if (e != cudaSuccess) rc = cuda_fail(e, "batched CG state");
                 continue;
             }
-            rc = restart(j, &O[j]);
+            rc = restart(j, rh + (size_t)(k % slots) * n3, &O[j]);
         }
         if (js.empty() && rc == LQCD_OK)
             for (int j = 0; j < n; ++j)
@@ -848,10 +852,8 @@ int mrhs_cg_core(lqcd_ctx *c, double mass, const double *sigma, int n, double to
     if (rc) return rc;
     // rr[j] is the residual of the x_j returned, but for a field whose iteration
     // was given up without a halt
-    std::vector<int> open;
     for (int j = 0; j < n; ++j)
-        if (done[j] == 2) open.push_back(j);
-    if (!open.empty() && (st = true_res(open, rr))) return st;
+        if (done[j] == 2 && (st = true_res(&j, 1, rr))) return st;
     int status = LQCD_OK;
     for (int j = 0; j < n; ++j) {
         const double res_j = b2[j] > 0 ? std::sqrt(rr[j] / b2[j]) : 0.0;
