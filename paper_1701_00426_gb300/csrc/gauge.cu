@@ -200,17 +200,26 @@ struct LinkRing {
     float2 e[D + 1][9][kGaugeThreads];   // slot D: the link that every side takes
 };
 
+// Element 0 of U_dir at a site in an array of link layout.  64 bits: the last
+// component of a lattice of 2^26 even sites lies beyond 2^32.
+__host__ __device__ constexpr size_t link_offset(int dir, int par, int idx, int Vh)
+{
+    return (size_t)((dir * 2 + par) * 9) * (size_t)Vh + (size_t)idx;
+}
+static_assert(link_offset(3, 1, (1 << 30) - 1, 1 << 30) + 8 * (size_t)(1 << 30) == ((size_t)72 << 30) - 1,
+              "the largest lattice that lqcd_create takes");
+
 // U_dir at a site into slot (one group; an empty one if !live)
 __device__ __forceinline__ void ring_fetch(LinkRing &R, int slot, const float2 *__restrict__ L, int dir, SiteIdx s, int Vh,
                                            bool live = true)
 {
     if (live) {
-        const unsigned off = ((unsigned)((dir * 2 + s.par) * 9) * (unsigned)Vh + (unsigned)s.idx);
+        const float2 *p = L + link_offset(dir, s.par, s.idx, Vh);
         const unsigned d = (unsigned)__cvta_generic_to_shared(&R.e[slot][0][threadIdx.x]);
 #pragma unroll
         for (int c = 0; c < 9; ++c)
             asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d + c * (unsigned)(kGaugeThreads * sizeof(float2))),
-                         "l"(L + (size_t)c * Vh + off), "n"
+                         "l"(p + (size_t)c * Vh), "n"
                          (sizeof(float2))
                          : "memory");
     }
