@@ -243,12 +243,6 @@ __device__ __forceinline__ void finalize_pq_shifts(SolverState *st, const PqCarr
     st->alpha_s_df[lane] = split_scalar(c.alpha * zn / c.zc);
 }
 
-__device__ inline void finalize_pq_warp(SolverState *st, double pq)
-{
-    const PqCarry c = finalize_pq_alpha(st, pq);
-    finalize_pq_shifts(st, c);
-}
-
 // The finaliser of K2's last block: alpha and, unless a block of K3 does it,
 // the shifted coefficients.
 __device__ __forceinline__ void finalize_pq_job(const IterJob &J, double pq)
