@@ -1084,8 +1084,8 @@ __device__ __forceinline__ const T *mom_ptr(const T *m, int mu, int P, int Vh)
 // links' way from L2 bounds it (some 75 links of 72 bytes per link in FP32, at
 // eleven warps per SM); through the ring their latency is spent under the
 // products, and L1's data path bounds it (81 % busy: in and out of the ring).
-// FP32, one GB300: 32^4 2180 -> 1837 us, 24^4 703 -> 621, 16^4 140 -> 131, a step
-// at 8^4 24.8 -> 22.8.  (One direction per block, no ring: 24^4 862.)  Rings of
+// FP32, one GB300: 32^4 2180 -> 1858 us, 24^4 703 -> 625, 16^4 140 -> 131, a step
+// at 8^4 24.8 -> 22.8 (of which 64-bit offsets 21 and 4 us).  (One direction per block, no ring: 24^4 862.)  Rings of
 // three and four slots, three and four blocks per SM: 24^4 626 / 621 and 621 /
 // 636; some links through the ring and some straight: 619 to 679, slower at
 // 32^4; bodies of their own for s = -1 and s = +1, without selections, outgrow the
