@@ -134,10 +134,14 @@ void prefault_host(void *p, size_t bytes)
     // Pages made writable without a write: the caller keeps what the buffer holds
     // if the call fails before its copy.  (An atomic OR with 0 also does that, but
     // its read maps the zero page first: 73 ms instead of 5 on Arm.)  A kernel
-    // that refuses leaves the faults to the copy.
+    // that refuses leaves the faults to the copy.  Four threads, 1 MB at a time: 191 MB
+    // in 1.9 ms; their whole share at a time 2.2, one thread 5.7, eight 5.7 (they
+    // share the address space's lock).
+    constexpr size_t kPiece = (size_t)1 << 20;
     auto touch = [=](size_t lo, size_t hi) {
-        const uintptr_t from = ((uintptr_t)p + lo) & ~(uintptr_t)(page - 1);
-        madvise((void *)from, (uintptr_t)p + hi - from, MADV_POPULATE_WRITE);
+        const uintptr_t end = (uintptr_t)p + hi;
+        for (uintptr_t a = ((uintptr_t)p + lo) & ~(uintptr_t)(page - 1); a < end; a += kPiece)
+            if (madvise((void *)a, std::min(kPiece, (size_t)(end - a)), MADV_POPULATE_WRITE) != 0) return;
     };
     const unsigned hw = std::thread::hardware_concurrency();
     const size_t nt = std::min({(size_t)4, (size_t)std::max(1u, hw / 2), bytes / kMin});

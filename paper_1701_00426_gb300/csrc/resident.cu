@@ -225,7 +225,7 @@ int resident_run(lqcd_ctx *c, const IterBatch<NJ> &B, int vp, int lf, int max_it
     LQCD_CUDA(cudaEventCreateWithFlags(&ev[1], cudaEventDisableTiming));
     auto enqueue = [&](int sl) -> cudaError_t {
         // a fresh range of tags for every launch, 0 left out (the cleared buffer);
-        // when they start again, no sum of the first round may be left
+        // when they start again, no sum of the first 2^32 may be left
         const bool wrap = c->res_tag > 0xFFFF0000u;
         if (wrap) c->res_tag = 0;
         R.tag0 = c->res_tag + 1;
